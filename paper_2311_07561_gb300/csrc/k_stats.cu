@@ -23,49 +23,65 @@ constexpr int kTX = 64;
 constexpr int kTY = 8;
 constexpr int kStatThreads = 256;   // each thread: x = tid % 64, y = tid / 64 and +4
 
+// Sum f and sum f^2 of the whole volume.  Bound by HBM: every thread keeps
+// four loads of 16 bytes in flight, sums in FP32 over 16 vectors (the same
+// partial sums for every launch of a volume) and only then in FP64, which on
+// this GPU runs at 1/64 of the FP32 rate.  The flush sits between two loops:
+// as a condition inside one loop it was evaluated for every vector, which
+// made the FP64 pipe the limit (256^3: 128 us, 0.5 TB/s).
+constexpr int kMomVec = 16;         // vectors per FP32 partial sum
+
+__device__ __forceinline__ void moments_add(float4& s1, float4& s2, const float4 v) {
+    s1.x += v.x; s1.y += v.y; s1.z += v.z; s1.w += v.w;
+    s2.x = fmaf(v.x, v.x, s2.x); s2.y = fmaf(v.y, v.y, s2.y);
+    s2.z = fmaf(v.z, v.z, s2.z); s2.w = fmaf(v.w, v.w, s2.w);
+}
+
 __global__ void __launch_bounds__(256) moments_kernel(const float* __restrict__ f, size_t n,
                                                       double* acc) {
-    __shared__ double r1[8], r2[8];
-    // float4 loads with four independent FP32 partial sums each, flushed to
-    // FP64 every 16 vectors; the scalar tail (n % 4, or an unaligned f) after
+    __shared__ double r1[256], r2[256];
     double d1 = 0.0, d2 = 0.0;
     const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     const size_t nthr = (size_t)gridDim.x * blockDim.x;
     const bool vec = ((uintptr_t)f & 15) == 0;
     const size_t n4 = vec ? n / 4 : 0;
     const float4* f4 = reinterpret_cast<const float4*>(f);
-    float4 s1 = make_float4(0.f, 0.f, 0.f, 0.f), s2 = s1;
-    int cntr = 0;
-    for (size_t i = tid; i < n4; i += nthr) {
-        const float4 v = __ldg(f4 + i);
-        s1.x += v.x; s1.y += v.y; s1.z += v.z; s1.w += v.w;
-        s2.x = fmaf(v.x, v.x, s2.x); s2.y = fmaf(v.y, v.y, s2.y);
-        s2.z = fmaf(v.z, v.z, s2.z); s2.w = fmaf(v.w, v.w, s2.w);
-        if (++cntr == 16) {
-            d1 += (double)s1.x + s1.y + s1.z + s1.w;
-            d2 += (double)s2.x + s2.y + s2.z + s2.w;
-            s1 = make_float4(0.f, 0.f, 0.f, 0.f); s2 = s1; cntr = 0;
+    size_t i = tid;
+#pragma unroll 1
+    while (i < n4) {
+        float4 s1 = make_float4(0.f, 0.f, 0.f, 0.f), s2 = s1;
+#pragma unroll 1
+        for (int c = 0; c < kMomVec && i < n4; c += 4, i += 4 * nthr) {
+            float4 v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                v[k] = i + k * nthr < n4 ? __ldg(f4 + i + k * nthr) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) moments_add(s1, s2, v[k]);
         }
+        d1 += (double)s1.x + s1.y + s1.z + s1.w;
+        d2 += (double)s2.x + s2.y + s2.z + s2.w;
     }
-    d1 += (double)s1.x + s1.y + s1.z + s1.w;
-    d2 += (double)s2.x + s2.y + s2.z + s2.w;
-    for (size_t i = 4 * n4 + tid; i < n; i += nthr) {
-        const float v = f[i];
+    // the scalar tail (n % 4, or all of an unaligned f)
+    for (size_t j = 4 * n4 + tid; j < n; j += nthr) {
+        const float v = f[j];
         d1 += v;
         d2 += (double)v * v;
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        d1 += __shfl_down_sync(0xffffffffu, d1, o);
-        d2 += __shfl_down_sync(0xffffffffu, d2, o);
+    // halving tree in shared memory: 255 FP64 additions a CTA, where shuffles
+    // in every warp would take 1280
+    r1[threadIdx.x] = d1;
+    r2[threadIdx.x] = d2;
+    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+        __syncthreads();
+        if (threadIdx.x < o) {
+            r1[threadIdx.x] += r1[threadIdx.x + o];
+            r2[threadIdx.x] += r2[threadIdx.x + o];
+        }
     }
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) { r1[wid] = d1; r2[wid] = d2; }
-    __syncthreads();
     if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) { a += r1[k]; b += r2[k]; }
-        atomicAdd(acc, a);
-        atomicAdd(acc + 1, b);
+        atomicAdd(acc, r1[0]);
+        atomicAdd(acc + 1, r2[0]);
     }
 }
 
