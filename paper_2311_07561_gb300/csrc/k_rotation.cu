@@ -9,7 +9,7 @@ static void fill_args(const RotBatch& b, const RotGrid& g, rot::SearchArgs& sa,
                       rot::PolishArgs& pa, const UnitList& list) {
     sa.b = b; pa.b = b;
     sa.list = list; pa.list = list;
-    sa.gm = g.d_m; sa.cell_end = g.d_cell_end; sa.n_grid = g.n_grid;
+    sa.gm = g.d_m; sa.cell_end = g.d_cell_end; sa.n_grid = g.n_grid; sa.n_cand = g.n_cand;
     pa.gq = g.d_q; pa.n_cand = g.n_cand; pa.newton = g.newton; pa.n_refine = g.n_refine;
 }
 

@@ -42,6 +42,7 @@ struct SearchArgs {
     const float* gm;        // n_grid x K4 (SIMT search)
     const int* cell_end;    // n_grid
     int n_grid;
+    int n_cand;             // candidates the refinement reads
 };
 
 struct PolishArgs {
