@@ -19,6 +19,7 @@
 #pragma once
 #include <cuda_bf16.h>
 
+#include "ttm_f2.cuh"
 #include "ttm_internal.h"
 
 namespace ttm {
@@ -345,6 +346,279 @@ __device__ void refine(const float (&C)[Geo<N>::K4], float sigma, int newton, fl
     lam_out = la;
 }
 
+// ---- two candidates at a time (orders 2 and 4) -----------------------------
+// The refinement is bound by the FMA pipe's register reads: scalar FMAs with
+// three different registers each ran at 78-86 lanes a clock and SM, packed
+// ones (fma.rn.f32x2, two FMAs per instruction) at 108.  So two candidates of
+// a voxel go through the evaluations together, one in each half of a register
+// pair; the components, which both share, are kept as pairs of equal halves
+// (2 K registers: orders 2 and 4 only, at order 6 they do not fit).  Every
+// half carries the operations of the scalar code in its order, so the results
+// are the same bits.
+template <int M>
+struct Monomials2 {
+    F2 v[n_comp(M) > 0 ? n_comp(M) : 1];
+};
+
+template <int M>
+__device__ __forceinline__ void monomials2(const F2 (&x)[4], Monomials2<M>& out) {
+    if constexpr (M == 0) {
+        out.v[0] = f2(1.0f, 1.0f);
+    } else if constexpr (M == 1) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out.v[k] = x[k];
+    } else {
+        Monomials2<M - 1> prev;
+        monomials2<M - 1>(x, prev);
+        constexpr MonoTab<M> T{};
+#pragma unroll
+        for (int k = 0; k < n_comp(M); ++k) out.v[k] = f2_mul(prev.v[T.parent[k]], x[T.var[k]]);
+    }
+}
+
+// a . b in the scalar code's order: a0 b0 + (a1 b1), then a2 b2, a3 b3
+__device__ __forceinline__ F2 f2_dot(const F2 (&a)[4], const F2 (&b)[4]) {
+    return f2_fma(a[3], b[3], f2_fma(a[2], b[2], f2_fma(a[0], b[0], f2_mul(a[1], b[1]))));
+}
+
+// grad_at for two points
+template <int N>
+__device__ __forceinline__ void grad2_at(const F2 (&C)[Geo<N>::K], const F2 (&x)[4], F2 (&g)[4],
+                                         F2& lam) {
+    constexpr GradTab<N> T{};
+    Monomials2<N - 1> mg;
+    monomials2<N - 1>(x, mg);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) g[i] = f2(0.f, 0.f);
+#pragma unroll
+    for (int b = 0; b < GradTab<N>::KG; ++b) {
+        const F2 mw = T.mult[b] == 1 ? mg.v[b]
+                                     : f2_mul(f2((float)T.mult[b], (float)T.mult[b]), mg.v[b]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) g[i] = f2_fma(mw, C[T.comp[i][b]], g[i]);
+    }
+    lam = f2_dot(x, g);
+}
+
+// eval_at for two points; h = the 10 entries of H
+template <int N>
+__device__ __forceinline__ void eval2_at(const F2 (&C)[Geo<N>::K], const F2 (&x)[4], F2 (&h)[10],
+                                         F2 (&g)[4], F2& lam) {
+    constexpr HessTab<N> T{};
+    Monomials2<N - 2> mb;
+    monomials2<N - 2>(x, mb);
+#pragma unroll
+    for (int p = 0; p < 10; ++p) h[p] = f2(0.f, 0.f);
+#pragma unroll
+    for (int b = 0; b < HessTab<N>::KB; ++b) {
+        const F2 mw = T.mult[b] == 1 ? mb.v[b]
+                                     : f2_mul(f2((float)T.mult[b], (float)T.mult[b]), mb.v[b]);
+#pragma unroll
+        for (int p = 0; p < 10; ++p) h[p] = f2_fma(mw, C[T.comp[p][b]], h[p]);
+    }
+    // rows of the symmetric matrix stored as pairs i <= j
+    const F2 H[4][4] = {{h[0], h[1], h[2], h[3]}, {h[1], h[4], h[5], h[6]},
+                        {h[2], h[5], h[7], h[8]}, {h[3], h[6], h[8], h[9]}};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) g[i] = f2_dot(H[i], x);
+    lam = f2_dot(g, x);
+}
+
+// the next power step's point from (x, g): normalise(g + sigma x)
+static __device__ __forceinline__ void power_point(const float (&g)[4], float sigma, const float (&x)[4],
+                                                   float (&out)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) out[i] = g[i] + sigma * x[i];
+    normalise4(out);
+}
+
+// power_steps for two candidates
+template <int N>
+__device__ __forceinline__ void power_steps2(const F2 (&C)[Geo<N>::K], float sigma, float (&xa)[4],
+                                             float (&xb)[4], float& la, float& lb, bool want_lam) {
+    F2 x[4], g[4], lam;
+#pragma unroll 1
+    for (int s = 0; s < 3; ++s) {
+        if (s == 2 && !want_lam) break;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = f2(xa[i], xb[i]);
+        grad2_at<N>(C, x, g, lam);
+        if (s == 2) break;
+        float ga[4], gb[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            ga[i] = f2_get(g[i], 0);
+            gb[i] = f2_get(g[i], 1);
+        }
+        power_point(ga, sigma, xa, xa);
+        power_point(gb, sigma, xb, xb);
+    }
+    la = f2_get(lam, 0);
+    lb = f2_get(lam, 1);
+}
+
+// one point's state through refine: the last accepted point, its gradient and
+// value, and the trial
+struct RefineState {
+    float xa[4], ga[4], xt[4], la;
+    bool trial_newton;
+};
+
+// what refine does with the evaluation (h, g, lam) of the trial
+template <int N>
+__device__ __forceinline__ void refine_step(RefineState& r, const float (&h)[10],
+                                            const float (&g)[4], float lam, float sigma, float eps,
+                                            bool last) {
+    if (r.trial_newton && lam < r.la - eps) {
+        if (last) return;
+        power_point(r.ga, sigma, r.xa, r.xt);
+        r.trial_newton = false;
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        r.xa[i] = r.xt[i];
+        r.ga[i] = g[i];
+    }
+    r.la = lam;
+    if (last) return;
+    float H[4][4], eta[4];
+    unpack(h, H);
+    if (newton_dir<N>(H, r.ga, r.xa, r.la, sigma, eta)) {
+        const float en2 = eta[0] * eta[0] + eta[1] * eta[1] + eta[2] * eta[2] + eta[3] * eta[3];
+        const float clip = en2 > 0.0625f ? 0.25f * rsqrtf(en2) : 1.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) r.xt[i] = r.xa[i] + clip * eta[i];
+        r.trial_newton = true;
+        normalise4(r.xt);
+    } else {
+        power_point(r.ga, sigma, r.xa, r.xt);
+        r.trial_newton = false;
+    }
+}
+
+// refine for two points
+template <int N>
+__device__ __forceinline__ void refine2(const F2 (&C)[Geo<N>::K], float sigma, int newton,
+                                        RefineState& a, RefineState& b) {
+    const float eps = 1e-6f * sigma;
+    const int iters = 1 + newton;
+#pragma unroll 1
+    for (int it = 0; it < iters; ++it) {
+        const bool last = it + 1 == iters;
+        F2 x[4], h[10], g[4], lam;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = f2(a.xt[i], b.xt[i]);
+        eval2_at<N>(C, x, h, g, lam);
+        float hs[10], gs[4];
+#pragma unroll
+        for (int p = 0; p < 10; ++p) hs[p] = f2_get(h[p], 0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) gs[i] = f2_get(g[i], 0);
+        refine_step<N>(a, hs, gs, f2_get(lam, 0), sigma, eps, last);
+#pragma unroll
+        for (int p = 0; p < 10; ++p) hs[p] = f2_get(h[p], 1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) gs[i] = f2_get(g[i], 1);
+        refine_step<N>(b, hs, gs, f2_get(lam, 1), sigma, eps, last);
+    }
+}
+
+// keep the kRefine largest values with their points, sorted descending
+static __device__ __forceinline__ void keep_point(float (&kl)[kRefine], float (&kx)[kRefine][4], float l,
+                                                  float (&x)[4]) {
+#pragma unroll
+    for (int s = 0; s < kRefine; ++s) {
+        const bool up = l > kl[s];
+        const float tl = kl[s];
+        kl[s] = up ? l : kl[s];
+        l = up ? tl : l;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float tx = kx[s][i];
+            kx[s][i] = up ? x[i] : kx[s][i];
+            x[i] = up ? tx : x[i];
+        }
+    }
+}
+
+template <int N> constexpr bool kPairs = N <= 4;
+
+// Refinement of a voxel's candidates, two at a time (orders 2 and 4); the
+// scalar loops of polish_kernel state the steps.
+template <int N>
+__device__ __forceinline__ void polish_pairs(const float (&Cs)[Geo<N>::K4], float score,
+                                             const uint32_t (&cw)[4], const PolishArgs& a,
+                                             float& best_l, float (&best_q)[4]) {
+    constexpr int K = Geo<N>::K;
+    F2 C[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) C[k] = f2(Cs[k], Cs[k]);
+    const float sigma = (float)(N - 1) * score;
+    best_l = -INFINITY;
+    const bool rank = a.n_cand > a.n_refine;
+    float kl[kRefine], kx[kRefine][4];
+#pragma unroll
+    for (int s = 0; s < kRefine; ++s) {
+        kl[s] = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) kx[s][i] = 0.f;
+    }
+    const int nc = a.n_cand < kMaxCand ? a.n_cand : kMaxCand;
+#pragma unroll 1
+    for (int k = 0; k < nc; k += 2) {
+        const uint32_t pair = k < 4 ? (k < 2 ? cw[0] : cw[1]) : (k < 6 ? cw[2] : cw[3]);
+        const int ia = (int)(pair & 0xFFFFu);
+        if (ia == 0xFFFF) break;
+        int ib = (int)(pair >> 16);
+        const bool two = k + 1 < nc && ib != 0xFFFF;
+        if (!two) ib = ia;
+        float xa[4], xb[4], la, lb;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            xa[i] = __ldg(a.gq + 4 * ia + i);
+            xb[i] = __ldg(a.gq + 4 * ib + i);
+        }
+        power_steps2<N>(C, sigma, xa, xb, la, lb, rank);
+        if (!rank) {
+            la = -(float)k;
+            lb = -(float)(k + 1);
+        }
+        keep_point(kl, kx, la, xa);
+        if (!two) break;
+        keep_point(kl, kx, lb, xb);
+    }
+#pragma unroll 1
+    for (int s = 0; s < kRefine; s += 2) {
+        if (s >= a.n_refine || !((s == 0 ? kl[0] : kl[2]) > -INFINITY)) break;
+        const bool two = s + 1 < a.n_refine && (s == 0 ? kl[1] : kl[3]) > -INFINITY;
+        RefineState ra, rb;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            // the kept points s and s + 1, picked with compile-time indices
+            ra.xt[i] = s == 0 ? kx[0][i] : kx[2][i];
+            rb.xt[i] = !two ? ra.xt[i] : (s == 0 ? kx[1][i] : kx[3][i]);
+            ra.xa[i] = ra.xt[i];
+            rb.xa[i] = rb.xt[i];
+            ra.ga[i] = rb.ga[i] = 0.f;
+        }
+        ra.la = rb.la = -INFINITY;
+        ra.trial_newton = rb.trial_newton = false;
+        refine2<N>(C, sigma, a.newton, ra, rb);
+        if (ra.la > best_l) {
+            best_l = ra.la;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) best_q[i] = ra.xa[i];
+        }
+        if (two && rb.la > best_l) {
+            best_l = rb.la;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) best_q[i] = rb.xa[i];
+        }
+    }
+    static_assert(kRefine == 4 && kMaxCand % 2 == 0, "points in pairs");
+}
+
 // Score and search: C_alpha = w Corr_alpha, score = ||C||_F, phi at every grid
 // point, best point of each region, the n_cand best regions -> candidate grid
 // indices (0xFFFF = none).  One thread per voxel; the grid table is staged in
@@ -416,10 +690,15 @@ __global__ void __launch_bounds__(kRotThreads) search_simt_kernel(const __grid_c
     store_candidates(sg.cand, i, ti, active);
 }
 
+// CTAs per SM the refinement's registers are sized for: four (128 registers)
+// in pairs, three (168) at order 6, whose K = 84 components fill more; at
+// order 8 (K = 165) the components alone take all there are
+template <int N> constexpr int polish_ctas() { return N <= 4 ? 4 : N == 6 ? 3 : 2; }
+
 // Refinement of the candidates and the outputs: lambda = the largest refined
 // phi, q its maximiser (canonical sign), C_alpha optionally.
 template <int N, typename CT>
-__global__ void __launch_bounds__(kRotThreads) polish_kernel(const __grid_constant__ PolishArgs a) {
+__global__ void __launch_bounds__(kRotThreads, polish_ctas<N>()) polish_kernel(const __grid_constant__ PolishArgs a) {
     constexpr int K = Geo<N>::K;
     constexpr int K4 = Geo<N>::K4;
     const RotSeg& sg = a.b.seg[seg_of(a.b, blockIdx.x)];
@@ -443,6 +722,9 @@ __global__ void __launch_bounds__(kRotThreads) polish_kernel(const __grid_consta
     float best_l = 0.f;
     float best_q[4] = {1.f, 0.f, 0.f, 0.f};
     if (score > 0.f && (cw[0] & 0xFFFFu) != 0xFFFFu) {
+        if constexpr (kPairs<N>) {
+            polish_pairs<N>(C, score, cw, a, best_l, best_q);
+        } else {
         const float sigma = (float)(N - 1) * score;
         best_l = -INFINITY;
         // phase 1: two power steps from every candidate; the kRefine best
@@ -503,6 +785,7 @@ __global__ void __launch_bounds__(kRotThreads) polish_kernel(const __grid_consta
 #pragma unroll
                 for (int i = 0; i < 4; ++i) best_q[i] = x[i];
             }
+        }
         }
         // canonical representative of {q, -q}: first non-zero component positive
         float sgn = 1.f;
