@@ -1085,19 +1085,40 @@ ttm_status ttm_build_tensor_template(const float* d_template, const float* d_mas
     cudaStream_t st = (cudaStream_t)stream;
     long long cnt = 0;
     char* ws = (char*)d_workspace;
-    double* d_msum = (double*)ws;
     int* d_bad = (int*)(ws + 8);
     float* rot = (float*)(ws + kHeader);
     TTM_CUDA_TRY(cudaMemsetAsync(ws, 0, kHeader, st));
-    TTM_TRY(launch_mask_sum(d_mask, s, d_msum, st, &cnt));
-    double msum = 0.0;
-    TTM_CUDA_TRY(cudaMemcpyAsync(&msum, d_msum, sizeof(double), cudaMemcpyDeviceToHost, st));
-    TTM_CUDA_TRY(cudaStreamSynchronize(st));
-    if (!(msum > 0.0)) return TTM_ERR_INVALID_ARG;
     const int nj = build_chunk(s, n_rot);
     const int s3 = s * s * s;
+    // the mask's voxels only, where the workspace has room for their list and
+    // tables beside the rotated copies (the copies shrink by the voxels left
+    // out), else every voxel of the box
+    const size_t area = (size_t)nj * s3;
+    const bool prepass = build_prepass_fits(s, area);
+    if (prepass)
+        TTM_TRY(launch_build_prepass(d_template, d_mask, s, ws, rot, area, st, &cnt));
+    else
+        TTM_TRY(launch_mask_sum(d_mask, s, (double*)ws, st, &cnt));
+    alignas(8) char head[64];
+    TTM_CUDA_TRY(cudaMemcpyAsync(head, ws, sizeof(head), cudaMemcpyDeviceToHost, st));
+    TTM_CUDA_TRY(cudaStreamSynchronize(st));
+    double msum = 0.0;
+    std::memcpy(&msum, head, sizeof(msum));
+    if (!(msum > 0.0)) return TTM_ERR_INVALID_ARG;
+    TemplateBuild tb;
+    const bool listed = prepass && build_layout(head, d_mask, s, n_order, nj, rot, area, &tb);
+    if (listed) {
+        TTM_TRY(launch_build_cells(tb, d_template, st, &cnt));
+        // voxels outside the mask
+        TTM_CUDA_TRY(cudaMemsetAsync(d_components, 0, (size_t)n_comp(n_order) * s3 * sizeof(float), st));
+    }
     for (int j0 = 0; j0 < n_rot; j0 += nj) {
         const int cnt_j = std::min(nj, n_rot - j0);
+        if (listed) {
+            TTM_TRY(launch_build_nodes(tb, n_order, d_quats, d_weights, n_rot, j0, cnt_j, d_components,
+                                       d_bad, st, &cnt));
+            continue;
+        }
         TTM_TRY(launch_rotate_normalise(d_template, d_mask, s, d_quats, j0, cnt_j, rot, msum, d_bad,
                                         st, &cnt));
         TTM_TRY(launch_fold_components(n_order, d_quats, d_weights, n_rot, j0, cnt_j, rot, s3,

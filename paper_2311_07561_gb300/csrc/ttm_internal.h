@@ -288,6 +288,27 @@ void build_grid_fp16(const float* m_rows, int K, int K4, int n_grid, std::vector
 bool search_tc_supported(int n_order, int n_grid, int n_cells);
 
 // tensor template build
+// Template build over the mask's voxels (k_template.cu): the split of the
+// workspace behind its header.
+struct TemplateBuild {
+    int s = 0, n = 0, soft = 0;           // box edge, mask voxels, mask values in (0, 1)
+    const float* mask = nullptr;
+    double mask_sum = 0.0;
+    int* list = nullptr;                  // mask voxels, packed coordinates
+    float* cells = nullptr;               // bordered template, four taps per cell
+    float2* norm = nullptr;               // offset and scale per node
+    float* coef = nullptr;                // w_j q_j^alpha per node
+    float* rot = nullptr;                 // samples, n per node
+};
+bool build_prepass_fits(int s, size_t area_floats);
+ttm_status launch_build_prepass(const float* t, const float* m, int s, void* head, float* area,
+                                size_t area_floats, cudaStream_t st, long long* cnt);
+bool build_layout(const void* head_host, const float* m, int s, int n_order, int nj, float* area,
+                  size_t area_floats, TemplateBuild* out);
+ttm_status launch_build_cells(const TemplateBuild& b, const float* t, cudaStream_t st, long long* cnt);
+ttm_status launch_build_nodes(const TemplateBuild& b, int n_order, const float* quats,
+                              const float* weights, int n_rot, int j0, int nj, float* comp,
+                              int* d_bad, cudaStream_t st, long long* cnt);
 ttm_status launch_rotate_normalise(const float* t, const float* m, int s, const float* quats,
                                    int j0, int nj, float* out, double mask_sum, int* d_bad,
                                    cudaStream_t st, long long* cnt);
