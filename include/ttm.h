@@ -121,7 +121,7 @@ typedef struct ttm_plan_opts {
     int rotation_chunks; /* split the interior into this many chunks and run  */
                          /* the search of chunk i+1 (high-priority stream)    */
                          /* beside the refinement of chunk i (low priority);  */
-                         /* 0 = default (8), 1 = one search then one refinement */
+                         /* 0 = default (1): one search, then one refinement     */
     float lowpass_sigma; /* > 0: the volume is prefiltered by a Gaussian of   */
                          /* this sigma (voxels, <= 7.9; ttm_lowpass) inside   */
                          /* ttm_local_stats, ttm_correlate, ttm_match_peaks;  */

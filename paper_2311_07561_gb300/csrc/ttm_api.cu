@@ -425,8 +425,13 @@ void free_plan(ttm_plan_s* P) {
 }
 
 // Streams and events of the pipelined rotation stage (rotation_chunks > 1).
+// The default is one chunk: since the search fills its SM by itself (ALU 73%
+// with its roles in separate warps) running it beside the refinement gains
+// nothing (256^3 order 4: 10.07 ms in one chunk, 10.20 in eight; 928x464x232
+// order 6: 55.14, 55.24), and small volumes save the launches (130x121x97:
+// 4.13, 4.23).
 ttm_status make_rotation_streams(ttm_plan_s* P) {
-    const int nch = P->opts.rotation_chunks > 0 ? P->opts.rotation_chunks : 8;
+    const int nch = P->opts.rotation_chunks > 0 ? P->opts.rotation_chunks : 1;
     if (nch > 64) return TTM_ERR_INVALID_ARG;
     P->rot_chunks = nch;
     if (nch == 1) return TTM_OK;
