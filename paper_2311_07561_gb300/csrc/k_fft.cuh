@@ -28,14 +28,29 @@
 namespace ttm {
 
 struct FftGeom {
-    int Xp, Yp, Zp, Xh;
+    int Xp, Yp, Zp, Xh;      // Xh: row length of the half spectrum (spec_pitch)
 };
 
 // Lines of a column pass: plane p = p0 + blockIdx.y (or the persistent tile's
-// plane) is plane z0 + (p % nz) of item p / nz, items zstride planes apart;
+// plane) is plane z0 + (p % nz), modulo zstride, of item p / nz, items zstride planes apart;
 // line samples lo..hi are stored (the rest are computed and dropped).
 struct ColsMap {
     int p0, nz, zstride, z0, lo, hi;
+};
+
+// The samples a forward column pass reads: all of them (len = L), or the len
+// samples from -c on, modulo L, the others being zero (a template box placed
+// about the origin); a scale other than 1 multiplies what is stored.
+struct ColsIn {
+    int c, len;
+    float scale;
+};
+
+// A batch of s^3 boxes in place of the real volume: box k is transformed into
+// spectrum k as if it sat in a zero volume with its centre voxel c at the
+// origin.  Only the rows that meet it are read and written (s = 0: a volume).
+struct BoxIn {
+    int s, c, n;
 };
 
 namespace fftk {
@@ -279,33 +294,47 @@ template <int L>
 __global__ void __launch_bounds__(kFftThreads) rows_r2c_t(const float* __restrict__ f, int X, int Y,
                                                           int Z, FftGeom g, float2* __restrict__ out,
                                                           const float2* __restrict__ tw, int mode,
-                                                          double* __restrict__ moments) {
+                                                          double* __restrict__ moments, BoxIn box) {
     constexpr int NB = rows_nb<L>();
     constexpr int PITCH = NB + 1;
     constexpr int XH = L / 2 + 1;
     extern __shared__ float2 sm[];
     float2* A = sm;
     float2* B = sm + L * PITCH;
-    const int row0 = blockIdx.x * NB;
-    const int nrows = g.Yp * g.Zp;
+    const long long row0 = (long long)blockIdx.x * NB;
+    const long long nrows = box.s ? (long long)box.n * box.s * box.s : (long long)g.Yp * g.Zp;
     const float mean = mode ? (float)(moments[0] / ((double)X * Y * Z)) : 0.f;
     constexpr int PER = (NB * L + kFftThreads - 1) / kFftThreads;
     __shared__ long long row_in[NB];         // input offset of each row, -1 = zero row
+    __shared__ long long row_out[NB];        // its row of the spectra, -1 = none
     if (threadIdx.x < NB) {
-        const int row = row0 + threadIdx.x;
-        long long off = -1;
-        if (row < nrows) {
-            const int y = row % g.Yp, z = row / g.Yp;
+        const long long row = row0 + threadIdx.x;
+        long long off = -1, to = -1;
+        if (row < nrows && box.s) {
+            const int per = box.s * box.s;
+            const long long item = row / per;
+            const int u = (int)(row - item * per);
+            int y = u % box.s - box.c, z = u / box.s - box.c;
+            if (y < 0) y += g.Yp;
+            if (z < 0) z += g.Zp;
+            off = row * box.s;
+            to = (item * g.Zp + z) * g.Yp + y;
+        } else if (row < nrows) {
+            const int y = (int)(row % g.Yp), z = (int)(row / g.Yp);
             if (y < Y && z < Z) off = (long long)(((size_t)z * Y + y) * X);
+            to = row;
         }
         row_in[threadIdx.x] = off;
+        row_out[threadIdx.x] = to;
     }
     __syncthreads();
     float vv[PER];
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
         const int e = threadIdx.x + i * kFftThreads;
-        const int r = e / L, x = e % L;
+        const int r = e / L;
+        int x = e % L;
+        if (box.s) x += box.c - (x + box.c >= L ? L : 0);
         float v = 0.f;
         if (e < NB * L && x < X) {
             const long long off = row_in[r];
@@ -341,20 +370,23 @@ __global__ void __launch_bounds__(kFftThreads) rows_r2c_t(const float* __restric
     float2* res = fft_lines_t<L, NB, PITCH, -1>(A, B, tw);
     for (int e = threadIdx.x; e < NB * XH; e += blockDim.x) {
         const int r = e / XH, k = e % XH;
-        const int row = row0 + r;
-        if (row < nrows) out[(size_t)row * XH + k] = res[k * PITCH + r];
+        const long long row = row_out[r];
+        if (row >= 0) out[(size_t)row * spec_pitch(L) + k] = res[k * PITCH + r];
     }
 }
 
 __device__ __forceinline__ size_t cols_plane_base(const ColsMap& mp, size_t p, int L, int B) {
     const size_t item = p / (size_t)mp.nz;
     const size_t zz = p - item * (size_t)mp.nz;
-    return (item * (size_t)mp.zstride + (size_t)mp.z0 + zz) * (size_t)L * (size_t)B;
+    size_t z = (size_t)mp.z0 + zz;
+    if (z >= (size_t)mp.zstride) z -= (size_t)mp.zstride;        // a box about the origin
+    return (item * (size_t)mp.zstride + z) * (size_t)L * (size_t)B;
 }
 
 template <int L, int SIGN, typename PS>
 __global__ void __launch_bounds__(kFftThreads) cols_t(PS* __restrict__ data, int B,
-                                                      const float2* __restrict__ tw, ColsMap mp) {
+                                                      const float2* __restrict__ tw, ColsMap mp,
+                                                      ColsIn ci) {
     constexpr int TB = cols_tb_s<L, PS>();
     extern __shared__ float2 sm[];
     float2* P = sm;
@@ -368,7 +400,9 @@ __global__ void __launch_bounds__(kFftThreads) cols_t(PS* __restrict__ data, int
     for (int i = 0; i < PER; ++i) {          // all loads in flight before any store
         const int e = threadIdx.x + i * kFftThreads;
         const int l = e / TB, bb = e & (TB - 1);
-        v[i] = (e < L * TB && bb < tb) ? ldc(data + base + (size_t)l * B + b0 + bb) : make_float2(0.f, 0.f);
+        // sample l of the box: (l + c) mod L below its length
+        const bool in = l + ci.c - (l + ci.c >= L ? L : 0) < ci.len;
+        v[i] = (e < L * TB && bb < tb && in) ? ldc(data + base + (size_t)l * B + b0 + bb) : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
@@ -381,61 +415,10 @@ __global__ void __launch_bounds__(kFftThreads) cols_t(PS* __restrict__ data, int
     for (int i = 0; i < PER; ++i) {
         const int e = threadIdx.x + i * kFftThreads;
         const int l = e / TB, bb = e & (TB - 1);
-        if (e < L * TB && bb < tb && l >= mp.lo && l <= mp.hi)
-            stc(data + base + (size_t)l * B + b0 + bb, res[e]);
-    }
-}
-
-// The same pass for long lines (one or two CTAs per SM): persistent CTAs walk
-// the (column tile, plane) tiles with a stride of gridDim.x, and the raw
-// elements of the next tile are loaded into registers while the current one
-// is transformed, so loads stay in flight through the Stockham stages.
-template <int L, int SIGN, typename PS>
-__global__ void __launch_bounds__(kFftThreads, 1) cols_pf_t(PS* __restrict__ data, int B,
-                                                            const float2* __restrict__ tw,
-                                                            ColsMap mp, int ntb, size_t ntiles) {
-    constexpr int TB = cols_tb_s<L, PS>();
-    extern __shared__ float2 sm[];
-    float2* P = sm;
-    float2* Q = sm + L * TB;
-    constexpr int PER = (L * TB + kFftThreads - 1) / kFftThreads;
-    PS nv[PER];
-    auto load = [&](size_t tile) {
-        const size_t plane = tile / (size_t)ntb;
-        const int b0 = (int)(tile - plane * (size_t)ntb) * TB;
-        const size_t base = cols_plane_base(mp, (size_t)mp.p0 + plane, L, B);
-        const int tb = min(TB, B - b0);
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int e = threadIdx.x + i * kFftThreads;
-            const int l = e / TB, bb = e & (TB - 1);
-            if (e < L * TB && bb < tb) nv[i] = data[base + (size_t)l * B + b0 + bb];
-        }
-    };
-    size_t tile = blockIdx.x;
-    if (tile >= ntiles) return;
-    load(tile);
-    for (; tile < ntiles; tile += gridDim.x) {
-        const size_t plane = tile / (size_t)ntb;
-        const int b0 = (int)(tile - plane * (size_t)ntb) * TB;
-        const size_t base = cols_plane_base(mp, (size_t)mp.p0 + plane, L, B);
-        const int tb = min(TB, B - b0);
-        __syncthreads();                      // the previous tile's result is stored
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int e = threadIdx.x + i * kFftThreads;
-            const int bb = e & (TB - 1);
-            if (e < L * TB) P[e] = bb < tb ? ldc(&nv[i]) : make_float2(0.f, 0.f);
-        }
-        if (tile + gridDim.x < ntiles) load(tile + gridDim.x);
-        __syncthreads();
-        float2* res = fft_lines_t<L, TB, TB, SIGN>(P, Q, tw);
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int e = threadIdx.x + i * kFftThreads;
-            const int l = e / TB, bb = e & (TB - 1);
-            if (e < L * TB && bb < tb && l >= mp.lo && l <= mp.hi)
-                stc(data + base + (size_t)l * B + b0 + bb, res[e]);
+        if (e < L * TB && bb < tb && l >= mp.lo && l <= mp.hi) {
+            float2 o = res[e];
+            if (ci.scale != 1.f) o = make_float2(o.x * ci.scale, o.y * ci.scale);
+            stc(data + base + (size_t)l * B + b0 + bb, o);
         }
     }
 }
@@ -574,7 +557,7 @@ template <int L>
 constexpr int c2r_stages_buffers() { return n_stages(L) >= 3 ? 2 : 1; }
 
 template <int L, typename PS>
-constexpr uint32_t c2r_tile_bytes() { return (uint32_t)(rows_nb<L>() * (L / 2 + 1) * sizeof(PS)); }
+constexpr uint32_t c2r_tile_bytes() { return (uint32_t)(rows_nb<L>() * spec_pitch(L) * sizeof(PS)); }
 
 template <int L>
 constexpr size_t c2r_fft_bytes() {
@@ -651,7 +634,7 @@ __global__ void __launch_bounds__(kFftThreads) rows_c2r_t(const PS* __restrict__
         const int zz = (int)(r / (size_t)nty);
         y_start = y_first + (int)(r - (size_t)zz * nty) * NB;
         z = keep.z0 + zz;
-        return in + ((item * (size_t)g.Zp + (size_t)z) * (size_t)g.Yp + (size_t)y_start) * XH;
+        return in + ((item * (size_t)g.Zp + (size_t)z) * (size_t)g.Yp + (size_t)y_start) * spec_pitch(L);
     };
     const uint32_t sbase = smem_addr(smraw);
     if (threadIdx.x == 0) {
@@ -713,8 +696,8 @@ __global__ void __launch_bounds__(kFftThreads) rows_c2r_t(const PS* __restrict__
         const int xk0 = keep.x0, xk1 = min(keep.x1, X - 1);
         stages_io<L, 0, NB, PITCH, +1>(
             [S](int x, int line) {
-                if (x < XH) return ldc(S + line * XH + x);
-                const float2 c = ldc(S + line * XH + (L - x));
+                if (x < XH) return ldc(S + line * spec_pitch(L) + x);
+                const float2 c = ldc(S + line * spec_pitch(L) + (L - x));
                 return make_float2(c.x, -c.y);
             },
             a, b,
@@ -731,6 +714,7 @@ __global__ void __launch_bounds__(kFftThreads) rows_c2r_t(const PS* __restrict__
 }  // namespace ttm
 
 #include "k_fft2.cuh"
+#include "k_fftp.cuh"
 
 namespace ttm {
 
@@ -742,9 +726,9 @@ namespace ttm {
 template <int L>
 struct FftLen {
     static cudaError_t rows_r2c(const float* f, int X, int Y, int Z, FftGeom g, float2* spec,
-                                const float2* tw, int mode, double* moments, cudaStream_t st);
+                                const float2* tw, int mode, double* moments, BoxIn box, cudaStream_t st);
     static cudaError_t cols(float2* d, int B, int na, ColsMap mp, const float2* tw, int sign,
-                            cudaStream_t st);
+                            ColsIn ci, cudaStream_t st);
     static cudaError_t cols_bf(__nv_bfloat162* d, int B, int na, ColsMap mp, const float2* tw,
                                int sign, cudaStream_t st);
     static cudaError_t cols_mul(const float2* spec, const float2* tspec, float2* prod, int Bz, int K,
@@ -768,26 +752,51 @@ inline cudaError_t sm_count(int* sms) {
     return cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
 }
 
-// lengths whose column tiles leave one CTA per SM take the persistent pass
-template <int L, typename PS>
-constexpr bool cols_persistent() { return 2 * (size_t)L * cols_tb_s<L, PS>() * sizeof(float2) > 100u * 1024u; }
-
 // persistent grid of a kernel: SMs x resident CTAs per SM, at most `work`
 template <class Kern>
-inline cudaError_t persistent_grid(Kern kern, size_t smem, size_t work, unsigned* grid) {
+inline cudaError_t persistent_grid(Kern kern, size_t smem, size_t work, unsigned* grid,
+                                  int threads = kTwoThreads) {
     int sms = 0, per_sm = 0;
     cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTwoThreads, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     if (e != cudaSuccess) return e;
     const size_t cap = (size_t)sms * (per_sm > 0 ? per_sm : 1);
     *grid = (unsigned)(work < cap ? work : cap);
     return cudaSuccess;
 }
 
+// column lengths that take the packed passes
+template <int L> constexpr bool cols_packed() { return TwoLevel<L>::L1 > 0; }
+template <int L, typename TS> constexpr bool mul_packed() {
+    if constexpr (TwoLevel<L>::L1 > 0) return MulPlan<L, TS>::on;
+    return false;
+}
+
 template <int L, int SIGN, typename PS>
-cudaError_t run_cols(PS* d, int B, int na, ColsMap mp, const float2* tw, cudaStream_t st) {
+cudaError_t run_cols(PS* d, int B, int na, ColsMap mp, const float2* tw, cudaStream_t st,
+                     ColsIn ci = ColsIn{0, L, 1.f}) {
+    if constexpr (cols_packed<L>()) {
+        constexpr int L1 = PackSplit<L>::L1, L2 = PackSplit<L>::L2;
+        constexpr int NP = 4;                    // 8 columns a tile
+        if (B % (2 * NP) == 0) {                 // rows of whole tiles (spec_pitch)
+            constexpr size_t smem = colsp_smem<L1, L2, NP, PS>(colsp_stages<L1, L2, NP, PS>());
+            auto kern = colsp_t<L1, L2, SIGN, NP, PS>;
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem);
+            if (e != cudaSuccess) return e;
+            const int ntb = B / (2 * NP);
+            const size_t ntiles = (size_t)ntb * na;
+            if (ntiles > 0xFFFFFFFFull) return cudaErrorInvalidValue;
+            unsigned grid = 0;
+            if ((e = persistent_grid(kern, smem, ntiles, &grid, L1 * NP)) != cudaSuccess) return e;
+            if (grid == 0) return cudaSuccess;
+            kern<<<grid, L1 * NP, smem, st>>>(d, B, tw, mp, ntb, (uint32_t)ntiles, ci);
+            return cudaGetLastError();
+        }
+    }
     if constexpr (two_level<L>()) {
+        if (ci.len != L || ci.scale != 1.f) return cudaErrorInvalidValue;     // box_cols_ok
         constexpr int L1 = TwoLevel<L>::L1, L2 = TwoLevel<L>::L2;
         constexpr int TB = kTwoThreads / L1;
         constexpr size_t smem = two_cols_smem<L1, L2>();
@@ -802,22 +811,10 @@ cudaError_t run_cols(PS* d, int B, int na, ColsMap mp, const float2* tw, cudaStr
         if (grid == 0) return cudaSuccess;
         kern<<<grid, kTwoThreads, smem, st>>>(d, B, tw, mp, ntb, ntiles);
         return cudaGetLastError();
-    }
-    constexpr int TB = cols_tb_s<L, PS>();
-    const size_t smem = (size_t)2 * L * TB * sizeof(float2);
-    const int ntb = (B + TB - 1) / TB;
-    if constexpr (cols_persistent<L, PS>()) {
-        cudaError_t e = cudaFuncSetAttribute(cols_pf_t<L, SIGN, PS>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int sms = 0;
-        if ((e = sm_count(&sms)) != cudaSuccess) return e;
-        const size_t ntiles = (size_t)ntb * na;
-        const unsigned grid = (unsigned)(ntiles < (size_t)sms ? ntiles : (size_t)sms);
-        if (grid == 0) return cudaSuccess;
-        cols_pf_t<L, SIGN, PS><<<grid, kFftThreads, smem, st>>>(d, B, tw, mp, ntb, ntiles);
-        return cudaGetLastError();
     } else {
+        constexpr int TB = cols_tb_s<L, PS>();
+        const size_t smem = (size_t)2 * L * TB * sizeof(float2);
+        const int ntb = (B + TB - 1) / TB;
         cudaError_t e = cudaFuncSetAttribute(cols_t<L, SIGN, PS>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -826,7 +823,7 @@ cudaError_t run_cols(PS* d, int B, int na, ColsMap mp, const float2* tw, cudaStr
             ColsMap m2 = mp;
             m2.p0 = mp.p0 + a0;
             dim3 grid(ntb, n);
-            cols_t<L, SIGN, PS><<<grid, kFftThreads, smem, st>>>(d, B, tw, m2);
+            cols_t<L, SIGN, PS><<<grid, kFftThreads, smem, st>>>(d, B, tw, m2, ci);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
         return cudaSuccess;
@@ -836,6 +833,27 @@ cudaError_t run_cols(PS* d, int B, int na, ColsMap mp, const float2* tw, cudaStr
 template <int L, typename TS, typename PS>
 cudaError_t run_cols_mul(const float2* spec, const TS* tspec, PS* prod, int Bz, int K,
                          const float2* tw, int lo, int hi, cudaStream_t st) {
+    if constexpr (mul_packed<L, TS>()) {
+        // one or two lines per column (the window sums): a CTA's teams would
+        // idle (144, one component: scalar 37 us, packed 44)
+        using Plan = MulPlan<L, TS>;
+        if (K > 2 && Bz % (2 * Plan::NP) == 0) {
+            constexpr int L1 = PackSplit<L>::L1, L2 = PackSplit<L>::L2, NP = Plan::NP, MS = Plan::MS;
+            constexpr size_t smem = mulp_smem<L1, L2, NP, MS, TS>();
+            constexpr int threads = L1 * NP * mulp_teams<L1, L2, NP, MS, TS>();
+            static_assert(threads > 0, "at least one team");
+            auto kern = mulp_t<L1, L2, NP, MS, TS, PS>;
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem);
+            if (e != cudaSuccess) return e;
+            int sms = 0;
+            if ((e = sm_count(&sms)) != cudaSuccess) return e;
+            const unsigned ntiles = (unsigned)(Bz / (2 * NP));
+            const unsigned grid = ntiles < (unsigned)sms ? ntiles : (unsigned)sms;
+            kern<<<grid, threads, smem, st>>>(spec, tspec, prod, Bz, K, tw, lo, hi, ntiles);
+            return cudaGetLastError();
+        }
+    }
     if constexpr (two_level<L>()) {
         constexpr int L1 = MulSplit<L>::L1, L2 = MulSplit<L>::L2;
         constexpr int TB = kTwoThreads / L1;
@@ -847,7 +865,7 @@ cudaError_t run_cols_mul(const float2* spec, const TS* tspec, PS* prod, int Bz, 
         dim3 grid((Bz + TB - 1) / TB, 1);
         kern<<<grid, kTwoThreads, smem, st>>>(spec, tspec, prod, Bz, K, tw, lo, hi);
         return cudaGetLastError();
-    }
+    } else {
     constexpr int TB = cols_tb<L>();
     const size_t smem = (size_t)2 * L * TB * sizeof(float2);
     cudaError_t e = cudaFuncSetAttribute(cols_mul_t<L, TS, PS>,
@@ -856,32 +874,41 @@ cudaError_t run_cols_mul(const float2* spec, const TS* tspec, PS* prod, int Bz, 
     dim3 grid((Bz + TB - 1) / TB, 1);
     cols_mul_t<L, TS, PS><<<grid, kFftThreads, smem, st>>>(spec, tspec, prod, Bz, K, tw, lo, hi);
     return cudaGetLastError();
+    }
 }
+
+// row lengths that take the packed pass: two-level ones below 960, where a
+// single CTA per SM is left (960: scalar 421 us, packed 438; 1024: 432, 740)
+template <int L> constexpr bool rows_packed() { return (c2r_half<L>() || two_level<L>()) && L < 960; }
 
 template <int L, typename PS, typename RT>
 cudaError_t run_rows_c2r(const PS* prod, int X, int Y, int Z, FftGeom g, RT* corr, int K,
                          const float2* tw, int* status, FftKeep keep, cudaStream_t st) {
-    if constexpr (c2r_half<L>()) {
-        constexpr int L1 = RowSplit<L / 2>::L1, L2 = RowSplit<L / 2>::L2;
-        constexpr int NR = kTwoThreads / L1 * c2r_groups<L1, L2, PS>();   // rows per tile
-        constexpr size_t smem = c2r_half_smem<L1, L2, PS>();
-        auto kern = rows_c2r_half_t<L1, L2, PS, RT>;
+    if constexpr (rows_packed<L>()) {
+        constexpr bool HALF = c2r_half<L>();
+        constexpr int L1 = HALF ? RowSplit<L / 2>::L1 : TwoLevel<L>::L1;
+        constexpr int L2 = HALF ? RowSplit<L / 2>::L2 : TwoLevel<L>::L2;
+        constexpr int NR = 2 * rowp_pairs<L1, L2>();                  // rows per tile
+        constexpr size_t smem = rowp_smem<L1, L2, HALF, PS>();
+        auto kern = rowsp_t<L1, L2, HALF, PS, RT>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e != cudaSuccess) return e;
         if (keep.z1 < keep.z0 || keep.y1 < keep.y0 || keep.x1 < keep.x0) return cudaSuccess;
         const size_t nrows = (size_t)K * (keep.z1 - keep.z0 + 1) * (keep.y1 - keep.y0 + 1);
         unsigned grid = 0;
-        if ((e = persistent_grid(kern, smem, (nrows + NR - 1) / NR, &grid)) != cudaSuccess) return e;
+        if ((e = persistent_grid(kern, smem, (nrows + NR - 1) / NR, &grid, kRowThreads)) != cudaSuccess)
+            return e;
         if (grid == 0) return cudaSuccess;
         (void)status;                       // no device-side waits in this pass
-        kern<<<grid, kTwoThreads, smem, st>>>(prod, X, Y, Z, g, corr, K, tw, keep);
+        kern<<<grid, kRowThreads, smem, st>>>(prod, X, Y, Z, g, corr, K, tw, keep);
         return cudaGetLastError();
-    } else if constexpr (two_level<L>()) {
-        constexpr int L1 = TwoLevel<L>::L1, L2 = TwoLevel<L>::L2;
-        constexpr int NR = kTwoThreads / L1;
-        constexpr size_t smem = two_rows_smem<L1, L2>();
-        auto kern = rows_c2r2_t<L1, L2, PS, RT>;
+    }
+    if constexpr (c2r_half<L>() && !rows_packed<L>()) {
+        constexpr int L1 = RowSplit<L / 2>::L1, L2 = RowSplit<L / 2>::L2;
+        constexpr int NR = kTwoThreads / L1 * c2r_groups<L1, L2, PS>();   // rows per tile
+        constexpr size_t smem = c2r_half_smem<L1, L2, PS>();
+        auto kern = rows_c2r_half_t<L1, L2, PS, RT>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e != cudaSuccess) return e;
@@ -919,7 +946,7 @@ cudaError_t run_rows_c2r(const PS* prod, int X, int Y, int Z, FftGeom g, RT* cor
 
 template <int L>
 cudaError_t FftLen<L>::rows_r2c(const float* f, int X, int Y, int Z, FftGeom g, float2* spec,
-                                const float2* tw, int mode, double* moments,
+                                const float2* tw, int mode, double* moments, BoxIn box,
                                 cudaStream_t st) {
     if constexpr (fftk::r2c_half<L>()) {
         constexpr int L1 = fftk::RowSplit<L / 2>::L1, L2 = fftk::RowSplit<L / 2>::L2;
@@ -929,12 +956,12 @@ cudaError_t FftLen<L>::rows_r2c(const float* f, int X, int Y, int Z, FftGeom g, 
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e != cudaSuccess) return e;
-        const size_t nrows = (size_t)g.Yp * g.Zp;
+        const size_t nrows = box.s ? (size_t)box.n * box.s * box.s : (size_t)g.Yp * g.Zp;
         unsigned grid = 0;
         if ((e = fftk::persistent_grid(kern, smem, (nrows + NR - 1) / NR, &grid)) != cudaSuccess)
             return e;
         if (grid == 0) return cudaSuccess;
-        kern<<<grid, fftk::kTwoThreads, smem, st>>>(f, X, Y, Z, g, spec, tw, mode, moments);
+        kern<<<grid, fftk::kTwoThreads, smem, st>>>(f, X, Y, Z, g, spec, tw, mode, moments, box);
         return cudaGetLastError();
     }
     constexpr int NB = fftk::rows_nb<L>();
@@ -942,17 +969,17 @@ cudaError_t FftLen<L>::rows_r2c(const float* f, int X, int Y, int Z, FftGeom g, 
     cudaError_t e = cudaFuncSetAttribute(fftk::rows_r2c_t<L>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int nrows = g.Yp * g.Zp;
-    fftk::rows_r2c_t<L><<<(nrows + NB - 1) / NB, fftk::kFftThreads, smem, st>>>(f, X, Y, Z, g, spec,
-                                                                               tw, mode, moments);
+    const long long nrows = box.s ? (long long)box.n * box.s * box.s : (long long)g.Yp * g.Zp;
+    fftk::rows_r2c_t<L><<<(unsigned)((nrows + NB - 1) / NB), fftk::kFftThreads, smem, st>>>(
+        f, X, Y, Z, g, spec, tw, mode, moments, box);
     return cudaGetLastError();
 }
 
 template <int L>
 cudaError_t FftLen<L>::cols(float2* d, int B, int na, ColsMap mp, const float2* tw, int sign,
-                            cudaStream_t st) {
-    return sign < 0 ? fftk::run_cols<L, -1, float2>(d, B, na, mp, tw, st)
-                    : fftk::run_cols<L, +1, float2>(d, B, na, mp, tw, st);
+                            ColsIn ci, cudaStream_t st) {
+    return sign < 0 ? fftk::run_cols<L, -1, float2>(d, B, na, mp, tw, st, ci)
+                    : fftk::run_cols<L, +1, float2>(d, B, na, mp, tw, st, ci);
 }
 
 template <int L>

@@ -339,104 +339,9 @@ __global__ void __launch_bounds__(kTwoThreads, mul_min_blocks<TS>(L2)) cols_mul2
     if constexpr (kAsync) cp_async_wait_all();
 }
 
-// ---- half-spectrum rows -> real x lines, two-level ------------------------
-// A tile is NR = 256 / L1 kept rows (z in keep.z0..z1, y in keep.y0..y1 of
-// every batch item, in that order); thread (row, n1) loads its L2 samples of
-// the Hermitian extension X[L - x] = conj X[x] straight from global memory;
-// the next tile's samples are loaded while the current one is transformed.
-// The real parts of the kept samples x0..x1 go to the X x Y x Z maps.
+// exchange bytes of the row passes
 template <int L1, int L2>
 constexpr size_t two_rows_smem() { return (size_t)(kTwoThreads / L1) * L2 * (L1 + 1) * sizeof(float2); }
-
-template <int L1, int L2, typename PS, typename RT>
-__global__ void __launch_bounds__(kTwoThreads, two_min_blocks<L2>()) rows_c2r2_t(const PS* __restrict__ in, int X,
-                                                              int Y, int Z, FftGeom g,
-                                                              RT* __restrict__ out, int n_batch,
-                                                              const float2* __restrict__ tw,
-                                                              FftKeep keep) {
-    constexpr int L = L1 * L2;
-    constexpr int XH = L / 2 + 1;
-    constexpr int NR = kTwoThreads / L1;
-    constexpr int ZP = L1 + 1;
-    extern __shared__ float2 zx[];                    // [row][k2][n1 (padded)]
-    const int t = threadIdx.x;
-    const int ra = t / L1, n1 = t % L1;
-    const int ny = keep.y1 - keep.y0 + 1, nz = keep.z1 - keep.z0 + 1;
-    const size_t nrows = (size_t)n_batch * nz * ny;
-    const size_t ntiles = (nrows + NR - 1) / NR;
-    // row q of the kept rows: its half-spectrum row and its output offset
-    auto row_of = [&](size_t q, size_t& src_row, long long& dst) {
-        const size_t per_item = (size_t)nz * ny;
-        const size_t item = q / per_item;
-        const size_t r = q - item * per_item;
-        const int z = keep.z0 + (int)(r / (size_t)ny);
-        const int y = keep.y0 + (int)(r % (size_t)ny);
-        src_row = (item * (size_t)g.Zp + (size_t)z) * (size_t)g.Yp + (size_t)y;
-        dst = (y < Y && z < Z) ? (long long)(item * ((size_t)X * Y * Z) + ((size_t)z * Y + y) * X)
-                               : -1;
-    };
-    PS raw[L2];
-    auto load = [&](size_t tile) {
-        const size_t q = tile * NR + ra;
-        if (q < nrows) {
-            size_t src;
-            long long dst;
-            row_of(q, src, dst);
-            const PS* rowp = in + src * XH;
-#pragma unroll
-            for (int n2 = 0; n2 < L2; ++n2) {
-                const int n = n1 + L1 * n2;
-                raw[n2] = rowp[n < XH ? n : L - n];
-            }
-        }
-    };
-    size_t tile = blockIdx.x;
-    if (tile >= ntiles) return;
-    load(tile);
-    const int xk0 = keep.x0, xk1 = min(keep.x1, X - 1);
-    for (; tile < ntiles; tile += gridDim.x) {
-        float2 v[L2];
-        const bool in_a = tile * NR + ra < nrows;
-#pragma unroll
-        for (int n2 = 0; n2 < L2; ++n2) {
-            const int n = n1 + L1 * n2;
-            float2 c = in_a ? ldc(&raw[n2]) : make_float2(0.f, 0.f);
-            if (n >= XH) c.y = -c.y;                   // conj X[L - n]
-            v[n2] = c;
-        }
-        if (tile + gridDim.x < ntiles) load(tile + gridDim.x);
-        dft_reg<L2, +1>(v);
-#pragma unroll
-        for (int k2 = 1; k2 < L2; ++k2) {
-            float2 w = __ldg(tw + n1 * k2);
-            w.y = -w.y;
-            v[k2] = cmul(v[k2], w);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k2 = 0; k2 < L2; ++k2) zx[(ra * L2 + k2) * ZP + n1] = v[k2];
-        __syncthreads();
-        for (int it = t; it < NR * L2; it += kTwoThreads) {
-            const int rb = it / L2, k2 = it % L2;
-            const size_t q = tile * NR + rb;
-            if (q >= nrows) continue;
-            size_t src;
-            long long dst;
-            row_of(q, src, dst);
-            float2 u[L1];
-#pragma unroll
-            for (int m = 0; m < L1; ++m) u[m] = zx[(rb * L2 + k2) * ZP + m];
-            dft_reg<L1, +1>(u);
-            if (dst >= 0) {
-#pragma unroll
-                for (int k1 = 0; k1 < L1; ++k1) {
-                    const int x = k2 + L2 * k1;
-                    if (x >= xk0 && x <= xk1) str(out + dst + x, u[k1].x);
-                }
-            }
-        }
-    }
-}
 
 // ---- half-spectrum rows -> real x lines through a half-length transform -----
 // A real line y[n] = sum_k X[k] W_L^(-n k) of even length L = 2M is the
@@ -538,7 +443,7 @@ __global__ void __launch_bounds__(kTwoThreads, two_min_blocks<L2>()) rows_c2r_ha
                 size_t src;
                 long long dst;
                 row_of(q, src, dst);
-                const PS* rowp = in + src * XH;
+                const PS* rowp = in + src * spec_pitch(2 * M);
 #pragma unroll
                 for (int n2 = 0; n2 < L2; ++n2) raw[h][n2] = rowp[n1 + L1 * n2];
                 xm[h] = rowp[M];
@@ -626,7 +531,7 @@ template <int L> constexpr bool r2c_half() { return L >= 256 && TwoLevel<L / 2>:
 template <int L1, int L2>
 __global__ void __launch_bounds__(kTwoThreads, two_min_blocks<L2>()) rows_r2c_half_t(
     const float* __restrict__ f, int X, int Y, int Z, FftGeom g, float2* __restrict__ out,
-    const float2* __restrict__ tw, int mode, double* __restrict__ moments) {
+    const float2* __restrict__ tw, int mode, double* __restrict__ moments, BoxIn box) {
     constexpr int M = L1 * L2;
     constexpr int XH = M + 1;
     constexpr int NR = kTwoThreads / L1;
@@ -635,14 +540,25 @@ __global__ void __launch_bounds__(kTwoThreads, two_min_blocks<L2>()) rows_r2c_ha
     __shared__ double part[kTwoThreads / 32];
     const int t = threadIdx.x;
     const int ra = t / L1, n1 = t % L1;
-    const size_t nrows = (size_t)g.Yp * g.Zp;
+    const size_t nrows = box.s ? (size_t)box.n * box.s * box.s : (size_t)g.Yp * g.Zp;
     const size_t ntiles = (nrows + NR - 1) / NR;
     const float mean = mode ? (float)(moments[0] / ((double)X * Y * Z)) : 0.f;
     // input offset of row q of the padded box, -1 for a zero row
     auto src_of = [&](size_t q) -> long long {
         if (q >= nrows) return -1;
+        if (box.s) return (long long)(q * box.s);
         const int y = (int)(q % (size_t)g.Yp), z = (int)(q / (size_t)g.Yp);
         return (y < Y && z < Z) ? (long long)(((size_t)z * Y + y) * X) : -1;
+    };
+    // its row of the spectra
+    auto dst_of = [&](size_t q) -> size_t {
+        if (!box.s) return q;
+        const size_t per = (size_t)box.s * box.s, item = q / per;
+        const int u = (int)(q - item * per);
+        int y = u % box.s - box.c, z = u / box.s - box.c;
+        if (y < 0) y += g.Yp;
+        if (z < 0) z += g.Zp;
+        return (item * g.Zp + z) * (size_t)g.Yp + y;
     };
     float q4 = 0.f;                                   // mode 2: this thread's sum of (f - mean)^4
     for (size_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -653,8 +569,15 @@ __global__ void __launch_bounds__(kTwoThreads, two_min_blocks<L2>()) rows_r2c_ha
             const int x = 2 * (n1 + L1 * n2);
             float a = 0.f, b = 0.f;
             if (sa >= 0) {
-                if (x < X) a = __ldg(f + sa + x) - mean;
-                if (x + 1 < X) b = __ldg(f + sa + x + 1) - mean;
+                if (box.s) {
+                    const int xa = x + box.c - (x + box.c >= 2 * M ? 2 * M : 0);
+                    const int xb = x + 1 + box.c - (x + 1 + box.c >= 2 * M ? 2 * M : 0);
+                    if (xa < X) a = __ldg(f + sa + xa);
+                    if (xb < X) b = __ldg(f + sa + xb);
+                } else {
+                    if (x < X) a = __ldg(f + sa + x) - mean;
+                    if (x + 1 < X) b = __ldg(f + sa + x + 1) - mean;
+                }
                 if (mode == 2) {
                     a *= a;
                     b *= b;
@@ -705,7 +628,7 @@ __global__ void __launch_bounds__(kTwoThreads, two_min_blocks<L2>()) rows_r2c_ha
             b.y = -b.y;                               // conj Z[M - k]
             const float2 e = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y + b.y));
             const float2 d = cmul(make_float2(0.5f * (a.x - b.x), 0.5f * (a.y - b.y)), __ldg(tw + k));
-            out[q * XH + k] = make_float2(e.x + d.y, e.y - d.x);      // e - i d
+            out[dst_of(q) * spec_pitch(2 * M) + k] = make_float2(e.x + d.y, e.y - d.x);      // e - i d
         }
     }
     if (mode == 2) {

@@ -217,17 +217,30 @@ __global__ void __launch_bounds__(256) peak_scan_kernel(
 }
 
 // Running maximum of c_j(x) = w(x) corr_j(x) over a batch of rotations j0..j0+nb-1
-// (Algorithm 1 reduced over the rotation set); first index wins ties.
-__global__ void best_rotation_kernel(const float* __restrict__ corr, int nb, int j0,
-                                     const float* __restrict__ w, size_t nvox,
-                                     float* __restrict__ best, int* __restrict__ best_j, int first) {
-    const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= nvox) return;
+// (Algorithm 1 reduced over the rotation set); first index wins ties.  Outside
+// the interior (where no correlation is computed) both outputs are 0.  Bound by
+// HBM: the nb maps are read once, eight loads in flight per thread.
+__global__ void __launch_bounds__(128) best_rotation_kernel(const float* __restrict__ corr, int nb, int j0,
+                                                            const float* __restrict__ w, int X, int Y,
+                                                            int Z, int s, float* __restrict__ best,
+                                                            int* __restrict__ best_j, int first) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y, z = blockIdx.z;
+    if (x >= X) return;
+    const size_t nvox = (size_t)X * Y * Z, v = ((size_t)z * Y + y) * X + x;
+    if (!(interior(x, X, s) && interior(y, Y, s) && interior(z, Z, s))) {
+        if (first) {
+            best[v] = 0.f;
+            best_j[v] = 0;
+        }
+        return;
+    }
     const float wv = w[v];
     float b = first ? -INFINITY : best[v];
     int bj = first ? 0 : best_j[v];
+#pragma unroll 8
     for (int j = 0; j < nb; ++j) {
-        const float c = wv * corr[(size_t)j * nvox + v];
+        const float c = wv * __ldg(corr + (size_t)j * nvox + v);
         if (c > b) { b = c; bj = j0 + j; }
     }
     best[v] = b;
@@ -236,11 +249,12 @@ __global__ void best_rotation_kernel(const float* __restrict__ corr, int nb, int
 
 }  // namespace
 
-ttm_status launch_best_rotation(const float* corr, int nb, int j0, const float* w, size_t nvox,
-                                float* best, int* best_j, bool first, cudaStream_t st,
+ttm_status launch_best_rotation(const float* corr, int nb, int j0, const float* w, int X, int Y, int Z,
+                                int s, float* best, int* best_j, bool first, cudaStream_t st,
                                 long long* cnt) {
-    best_rotation_kernel<<<(unsigned)((nvox + 255) / 256), 256, 0, st>>>(corr, nb, j0, w, nvox, best,
-                                                                          best_j, first ? 1 : 0);
+    if (Y > 65535 || Z > 65535) return TTM_ERR_UNSUPPORTED;
+    const dim3 grid((unsigned)((X + 127) / 128), (unsigned)Y, (unsigned)Z);
+    best_rotation_kernel<<<grid, 128, 0, st>>>(corr, nb, j0, w, X, Y, Z, s, best, best_j, first ? 1 : 0);
     return after_launch(cnt);
 }
 

@@ -462,7 +462,10 @@ constexpr size_t kProdBudget = (size_t)8 << 30;
 
 int comp_group(const ttm_plan_s* P, const ProblemData& pr) {
     const size_t per = pr.fft.nspec() * 2 * (pr.mixed ? 2 : 4);
-    const size_t g = per ? kProdBudget / per : (size_t)P->K;
+    size_t g = per ? kProdBudget / per : (size_t)P->K;
+    // whole rounds of the fused multiply's teams (2 to 8 per CTA take the
+    // components of a group in turn)
+    if (g < (size_t)P->K) g = g >= 12 ? g / 12 * 12 : g >= 3 ? g / 3 * 3 : g;
     return (int)std::max<size_t>(1, std::min<size_t>(g, (size_t)P->K));
 }
 
@@ -1533,6 +1536,8 @@ ttm_status ttm_classical_ncc(ttm_plan_t plan, int problem, const float* d_templa
     TTM_TRY(timed(plan, KC_FFT_FORWARD, st, [&] {
         return launch_fft_forward(d_vol, pr.X, pr.Y, pr.Z, pr.fft, spec, st, &plan->launches);
     }));
+    // the NCC is defined on the interior (w = 0 elsewhere)
+    const FftKeep keep = fft_keep_interior(pr.X, pr.Y, pr.Z, s);
     for (int j0 = 0; j0 < n_rot; j0 += kClassicalBatch) {
         const int nb = std::min(kClassicalBatch, n_rot - j0);
         TTM_TRY(timed(plan, KC_TEMPLATE, st, [&] {
@@ -1542,17 +1547,16 @@ ttm_status ttm_classical_ncc(ttm_plan_t plan, int problem, const float* d_templa
         }));
         TTM_TRY(timed(plan, KC_FFT_SPECTRUM, st, [&] {
             return launch_fft_spectrum_inverse_z(spec, tspec, nb, pr.fft, prod,
-                                                 fft_keep_all(pr.X, pr.Y, pr.Z), st,
+                                                 keep, st,
                                                  &plan->launches);
         }));
         TTM_TRY(timed(plan, KC_FFT_INVERSE, st, [&] {
             return launch_fft_inverse_yx(prod, nb, pr.X, pr.Y, pr.Z, pr.fft, maps,
-                                         (int*)(ws + 32), fft_keep_all(pr.X, pr.Y, pr.Z), st,
-                                         &plan->launches);
+                                         (int*)(ws + 32), keep, st, &plan->launches);
         }));
         TTM_TRY(timed(plan, KC_PEAKS, st, [&] {
-            return launch_best_rotation(maps, nb, j0, d_w, pr.nvox(), d_best, d_best_index, j0 == 0,
-                                        st, &plan->launches);
+            return launch_best_rotation(maps, nb, j0, d_w, pr.X, pr.Y, pr.Z, s, d_best, d_best_index,
+                                        j0 == 0, st, &plan->launches);
         }));
     }
     int bad = 0;

@@ -36,13 +36,22 @@ struct TemplateData {
     int spec_shape[3] = {0, 0, 0};
 };
 
+// Row length of a half spectrum: Xp / 2 + 1 samples, from 128 points up padded to
+// a multiple of 8, so that the column passes' tiles of 8 columns start on whole
+// 32-byte sectors at every storage type (the padding columns hold nothing in
+// use).  Shorter rows stay as they are: the padding would be up to a fifth of
+// them (64: rows_c2r 24 us, padded 34).
+__host__ __device__ constexpr int spec_pitch(int Xp) {
+    return Xp >= 128 ? ((Xp / 2 + 1) + 7) & ~7 : Xp / 2 + 1;
+}
+
 // Padded FFT box of a problem and its twiddle tables (plan-owned).
 struct FftShape {
     int Xp = 0, Yp = 0, Zp = 0;
     const float2* d_tw_x = nullptr;   // exp(-2 pi i k / Xp), k < Xp
     const float2* d_tw_y = nullptr;
     const float2* d_tw_z = nullptr;
-    size_t nspec() const { return (size_t)(Xp / 2 + 1) * Yp * Zp; }
+    size_t nspec() const { return (size_t)spec_pitch(Xp) * Yp * Zp; }
 };
 
 struct ProblemData {
@@ -154,7 +163,6 @@ inline FftKeep fft_keep_interior(int X, int Y, int Z, int s) {
     const int c = s / 2;
     return FftKeep{c, X - s + c, c, Y - s + c, c, Z - s + c};
 }
-inline FftKeep fft_keep_all(int X, int Y, int Z) { return FftKeep{0, X - 1, 0, Y - 1, 0, Z - 1}; }
 
 // Rotation search grid (device tables owned by the plan).
 struct RotGrid {
@@ -355,8 +363,8 @@ ttm_status launch_template_spectra(const float* comp, int K, int s, const FftSha
                                    float* pad, float2* tspec, cudaStream_t st, long long* cnt);
 
 // classical comparator
-ttm_status launch_best_rotation(const float* corr, int nb, int j0, const float* w, size_t nvox,
-                                float* best, int* best_j, bool first, cudaStream_t st,
+ttm_status launch_best_rotation(const float* corr, int nb, int j0, const float* w, int X, int Y, int Z,
+                                int s, float* best, int* best_j, bool first, cudaStream_t st,
                                 long long* cnt);
 
 // peaks
