@@ -542,15 +542,20 @@ __global__ void __launch_bounds__(128) stats_from_sums_kernel(
     int Y, int Z, int s, double mask_sum, const double* __restrict__ moments, double kappa,
     unsigned int* __restrict__ flagged) {
     __shared__ double sh[4];
-    if (threadIdx.x == 0) {
+    // one warp each for the chains of FP64 divisions and square roots, which
+    // take microseconds here
+    if ((threadIdx.x & 31) == 0) {
+        const int w = threadIdx.x >> 5;
         const double nv = (double)X * Y * Z;
-        const double mean = moments[0] / nv;
-        const double var_f = fmax(moments[1] / nv - mean * mean, 0.0);
         const double eps = 5.9604644775390625e-8;          // 2^-24
-        sh[0] = 1.0 / mask_sum;
-        sh[1] = 1e-6 * mask_sum * var_f;
-        sh[2] = kappa * eps * mask_sum * sqrt(var_f);       // bound on |dS1|
-        sh[3] = kappa * eps * mask_sum * sqrt(fmax(moments[2], 0.0) / nv);   // on |dS2|
+        if (w == 0) sh[0] = 1.0 / mask_sum;
+        if (w == 1 || w == 2) {
+            const double mean = moments[0] / nv;
+            const double var_f = fmax(moments[1] / nv - mean * mean, 0.0);
+            if (w == 1) sh[1] = 1e-6 * mask_sum * var_f;
+            else sh[2] = kappa * eps * mask_sum * sqrt(var_f);       // bound on |dS1|
+        }
+        if (w == 3) sh[3] = kappa * eps * mask_sum * sqrt(fmax(moments[2], 0.0) / nv);   // on |dS2|
     }
     __syncthreads();
     const float fim = (float)sh[0], ffl = (float)sh[1], fe1 = (float)sh[2], fe2 = (float)sh[3];

@@ -437,6 +437,9 @@ __global__ void __launch_bounds__(kFftThreads, 2) cols_mul_t(const float2* __res
     const int b0 = blockIdx.x * TB;
     const int tb = min(TB, B - b0);
     const size_t plane = (size_t)L * B;
+    // this CTA's share of the components
+    const int k0 = (int)((long long)K * blockIdx.y / gridDim.y);
+    const int k1 = (int)((long long)K * (blockIdx.y + 1) / gridDim.y);
     // this thread's elements of the image tile stay in registers
     float2 fi[PER];
 #pragma unroll
@@ -451,17 +454,17 @@ __global__ void __launch_bounds__(kFftThreads, 2) cols_mul_t(const float2* __res
     for (int i = 0; i < PER; ++i) {
         const int e = threadIdx.x + i * kFftThreads;
         const int l = e / TB, bb = e & (TB - 1);
-        tv[i] = (K > 0 && e < L * TB && bb < tb) ? ldgc(tspec + (size_t)l * B + b0 + bb)
+        tv[i] = (k0 < k1 && e < L * TB && bb < tb) ? ldgc(tspec + (size_t)k0 * plane + (size_t)l * B + b0 + bb)
                                                   : make_float2(0.f, 0.f);
     }
-    for (int k = 0; k < K; ++k) {
+    for (int k = k0; k < k1; ++k) {
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
             const int e = threadIdx.x + i * kFftThreads;
             if (e < L * TB) P[e] = cmulc(fi[i], tv[i]);
         }
-        if (k + 1 < K) {
+        if (k + 1 < k1) {
             const TS* ts = tspec + (size_t)(k + 1) * plane;
 #pragma unroll
             for (int i = 0; i < PER; ++i) {
@@ -871,7 +874,11 @@ cudaError_t run_cols_mul(const float2* spec, const TS* tspec, PS* prod, int Bz, 
     cudaError_t e = cudaFuncSetAttribute(cols_mul_t<L, TS, PS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((Bz + TB - 1) / TB, 1);
+    // small boxes: the components of a tile shared by several CTAs, up to four per SM
+    // (64^3 box, 35 components: 66 tiles)
+    const unsigned tiles = (unsigned)((Bz + TB - 1) / TB);
+    const unsigned parts = tiles >= 304 ? 1u : 608u / tiles;
+    const dim3 grid(tiles, parts < (unsigned)K ? parts : (unsigned)(K > 0 ? K : 1));
     cols_mul_t<L, TS, PS><<<grid, kFftThreads, smem, st>>>(spec, tspec, prod, Bz, K, tw, lo, hi);
     return cudaGetLastError();
     }

@@ -196,6 +196,131 @@ __global__ void __launch_bounds__(kStatThreads) local_stats_kernel(StatsArgs a) 
     }
 }
 
+// The same statistics for small masks (MarchMask), as the direct path has
+// them.  FP64 runs at 2 operations a clock and SM here, so what counts is how
+// few of them a voxel needs.  A CTA owns 32 x 8 columns and marches along z: of
+// each input plane it forms once, in shared memory, the sums over every
+// distinct x-window of the mask at every row; a voxel then adds one window sum
+// per run of each distinct mask plane (the planes dz and -dz of a ball are one)
+// and the plane's sum goes to the outputs z - dz that have it, kept in
+// registers until their last plane has passed.  About 140 FP64 operations per
+// voxel for a ball of radius 4, where prefix sums rebuilt for every output
+// plane took 690 (130 x 121 x 97, s = 9: 3022 us).
+struct MarchArgs {
+    StatsArgs s;
+    MarchMask m;
+    const int* runs;
+    int z0, z1, nzc;         // interior planes, planes per CTA
+    int x0, y0;              // first interior voxel
+};
+
+constexpr int kMarchX = 32, kMarchY = 8;
+
+template <int NDZ>
+__global__ void __launch_bounds__(kMarchX * kMarchY) march_stats_kernel(const __grid_constant__ MarchArgs a) {
+    extern __shared__ double smem[];
+    const int rows = kMarchY + (a.s.dy_max - a.s.dy_min);
+    const int width = kMarchX + (a.s.x_max - a.s.x_min);
+    double2* W = reinterpret_cast<double2*>(smem);                   // [window][row][x]
+    double* V = smem + (size_t)a.m.n_win * rows * kMarchX * 2;       // [row][width]
+    __shared__ double sh[2];
+    const int t = threadIdx.x, lx = t % kMarchX, ly = t / kMarchX;
+    const int x0 = a.x0 + blockIdx.x * kMarchX, y0 = a.y0 + blockIdx.y * kMarchY;
+    const int z0 = a.z0 + blockIdx.z * a.nzc, z1 = min(z0 + a.nzc - 1, a.z1);
+    if (t == 0) {
+        const double nvox = (double)a.s.X * a.s.Y * a.s.Z;
+        const double mean = a.s.moments[0] / nvox;
+        const double var_f = fmax(a.s.moments[1] / nvox - mean * mean, 0.0);
+        sh[0] = 1.0 / a.s.mask_sum;
+        sh[1] = 1e-6 * a.s.mask_sum * var_f;
+    }
+    // reference value near the middle of the tile (the variance does not
+    // change under a shift, which removes the cancellation of large offsets)
+    const double mu = __ldg(a.s.f + ((size_t)min((z0 + z1) / 2, a.s.Z - 1) * a.s.Y +
+                                     min(y0 + kMarchY / 2, a.s.Y - 1)) * a.s.X +
+                            min(x0 + kMarchX / 2, a.s.X - 1));
+    double s1[NDZ], s2[NDZ];                 // slot k: output plane zz - dz_min - k
+#pragma unroll
+    for (int k = 0; k < NDZ; ++k) s1[k] = s2[k] = 0.0;
+    for (int zz = z0 + a.s.dz_min; zz <= z1 + a.s.dz_max; ++zz) {
+        __syncthreads();
+        // zz lies in the volume: every output plane is interior
+        for (int e = t; e < rows * width; e += kMarchX * kMarchY) {
+            const int rr = e / width, i = e - rr * width;
+            const int yy = y0 + a.s.dy_min + rr, xx = x0 + a.s.x_min + i;
+            V[e] = yy < a.s.Y && xx < a.s.X
+                ? (double)__ldg(a.s.f + ((size_t)zz * a.s.Y + yy) * a.s.X + xx) - mu : 0.0;
+        }
+        __syncthreads();
+        for (int e = t; e < rows * kMarchX; e += kMarchX * kMarchY) {
+            const int rr = e / kMarchX, x = e % kMarchX;
+            const double* v = V + rr * width + x - a.s.x_min;      // v[dx]
+            int lo = 1, hi = 0;                                    // the window summed so far
+            double c1 = 0.0, c2 = 0.0;
+            for (int w = 0; w < a.m.n_win; ++w) {
+                const int w0 = a.m.x0[w], w1 = a.m.x1[w];
+                if (lo > hi || w0 > lo || w1 < hi) {               // not an extension
+                    c1 = c2 = 0.0;
+                    lo = w0;
+                    hi = w0 - 1;
+                }
+                while (lo > w0) { const double d = v[--lo]; c1 += d; c2 = fma(d, d, c2); }
+                while (hi < w1) { const double d = v[++hi]; c1 += d; c2 = fma(d, d, c2); }
+                W[(w * rows + rr) * kMarchX + x] = make_double2(c1, c2);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = NDZ - 1; k > 0; --k) {
+            s1[k] = s1[k - 1];
+            s2[k] = s2[k - 1];
+        }
+        s1[0] = s2[0] = 0.0;
+        for (int c = 0; c < a.m.n_cls; ++c) {
+            double p1 = 0.0, p2 = 0.0;
+            for (int k = a.m.run0[c]; k < a.m.run0[c + 1]; ++k) {
+                const int run = __ldg(a.runs + k);
+                const double2 q = W[((run >> 8) * rows + ly + (run & 255)) * kMarchX + lx];
+                p1 += q.x;
+                p2 += q.y;
+            }
+#pragma unroll
+            for (int k = 0; k < NDZ; ++k)
+                if (a.m.cls[k] == c) {
+                    s1[k] += p1;
+                    s2[k] += p2;
+                }
+        }
+        const int z = zz - a.s.dz_max;            // its last plane has passed
+        const int x = x0 + lx, y = y0 + ly;
+        if (z >= z0 && z <= z1 && interior(x, a.s.X, a.s.s) && interior(y, a.s.Y, a.s.s)) {
+            const double V2 = s2[NDZ - 1] - s1[NDZ - 1] * s1[NDZ - 1] * sh[0];
+            a.s.w[((size_t)z * a.s.Y + y) * a.s.X + x] = V2 > sh[1] ? rsqrtf((float)V2) : 0.f;
+        }
+    }
+}
+
+// w = 0 outside the interior
+__global__ void __launch_bounds__(256) exterior_zero_kernel(float* __restrict__ w, int X, int Y, int Z, int s) {
+    const int rows = Y * Z;
+    for (int r = blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8) {
+        const bool in = interior(r % Y, Y, s) && interior(r / Y, Z, s);
+        for (int x = threadIdx.x & 31; x < X; x += 32)
+            if (!in || !interior(x, X, s)) w[(size_t)r * X + x] = 0.f;
+    }
+}
+
+template <int NDZ>
+ttm_status march_launch(const MarchArgs& a, dim3 grid, size_t smem, int ndz, cudaStream_t st) {
+    if constexpr (NDZ > 1) {
+        if (ndz < NDZ) return march_launch<NDZ - 1>(a, grid, smem, ndz, st);
+    }
+    TTM_CUDA_TRY(cudaFuncSetAttribute(march_stats_kernel<NDZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)smem));
+    march_stats_kernel<NDZ><<<grid, kMarchX * kMarchY, smem, st>>>(a);
+    return TTM_OK;
+}
+
 // Exact local statistics at the voxels flagged by the FFT window sums (w = -1
 // there; flagged voxels are interior).  One warp per flagged voxel: the lanes
 // split the s^3 mask box and accumulate m (f - f(x)) and m (f - f(x))^2 in
@@ -293,6 +418,30 @@ ttm_status launch_local_stats(const float* f, int X, int Y, int Z, const Templat
     a.x_min = T.x_min; a.x_max = T.x_max;
     a.mask_sum = T.desc.mask_sum;
     a.moments = d_moments;
+    const VoxBox box = interior_box(X, Y, Z, T.desc.s);
+    if (T.march.n_win > 0 && box.count() > 0) {
+        // every output's planes lie in the volume (a mask reaches at most its
+        // box).  Planes per CTA: fewer cost more halo planes, more leave SMs
+        // idle; enough CTAs for two per SM, at least 8 planes
+        MarchArgs m;
+        m.s = a; m.m = T.march; m.runs = T.d_march_runs;
+        m.x0 = box.x0; m.y0 = box.y0; m.z0 = box.z0; m.z1 = box.z0 + (int)box.nz - 1;
+        const int gx = ((int)box.nx + kMarchX - 1) / kMarchX, gy = ((int)box.ny + kMarchY - 1) / kMarchY;
+        const int want = (304 + gx * gy - 1) / (gx * gy);
+        int nzc = ((int)box.nz + want - 1) / want;
+        nzc = nzc < 8 ? 8 : nzc > 64 ? 64 : nzc;
+        m.nzc = nzc;
+        const int ndz = T.dz_max - T.dz_min + 1;
+        const int rows = kMarchY + (T.dy_max - T.dy_min), width = kMarchX + (T.x_max - T.x_min);
+        const size_t smem = (size_t)rows * (T.march.n_win * kMarchX * 16 + width * 8);
+        const dim3 grid(gx, gy, ((int)box.nz + nzc - 1) / nzc);
+        if (gy <= 65535) {
+            exterior_zero_kernel<<<152 * 8, 256, 0, st>>>(w, X, Y, Z, T.desc.s);
+            TTM_TRY(after_launch(cnt));
+            TTM_TRY(march_launch<kMarchDz>(m, grid, smem, ndz, st));
+            return after_launch(cnt);
+        }
+    }
     const int rows = kTY + (T.dy_max - T.dy_min);
     const int pitch = kTX + (T.x_max - T.x_min) + 1;
     const size_t smem = (size_t)2 * rows * pitch * sizeof(double);

@@ -322,7 +322,7 @@ __device__ __forceinline__ float two_sum(float a, float b, float& e) {
 // and scale.  FP64 runs at 1/64 of the FP32 rate here, so the sums of four
 // samples (and of their exact squares) are formed in FP32 without error, sum
 // and remainder apart, and one FP64 addition takes the sum.
-__global__ void __launch_bounds__(kRotThreads) rotate_list_kernel(
+__global__ void __launch_bounds__(256, 5) rotate_list_kernel(
     const float4* __restrict__ cells, const float* __restrict__ m, int s,
     const float* __restrict__ quats, int j0, const int* __restrict__ list, int n, int soft,
     float* __restrict__ out, float2* __restrict__ norm, double mask_sum, int* bad) {
@@ -445,21 +445,33 @@ __global__ void __launch_bounds__(128) coef_kernel(const float* __restrict__ qua
 
 // T_alpha(u) over the listed voxels, A components (blockIdx.y) and V voxels per
 // thread: a coefficient pair read from shared memory (a broadcast) feeds V
-// packed FMAs of two components each.  Bound by the FMA pipe (packed: 116 FMAs
-// a clock and SM).  A component's sum runs over the nodes in order, as in
-// fold_kernel.
+// packed FMAs of two components each.  The samples, coefficients and norms of
+// the next 16 nodes are copied into shared memory while this step's are folded
+// (loading them into registers at the step's start left the FMA pipe idle two
+// thirds of the time: 30.5 ms at 64^3, order 6, 20000 rotations).  Bound by the
+// FMA pipe (packed: 116 FMAs a clock and SM).  A component's sum runs over the
+// nodes in order, as in fold_kernel.
 constexpr int kFold2Threads = 128;
 
+template <int A> constexpr int fold_ctas() { return A > 12 ? 3 : 6; }
+
+__device__ __forceinline__ void copy_async(void* dst, const void* src, int bytes) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if (bytes == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+    else if (bytes == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+}
+
 template <int A, int V>
-__global__ void __launch_bounds__(kFold2Threads) fold_list_kernel(
+__global__ void __launch_bounds__(kFold2Threads, fold_ctas<A>()) fold_list_kernel(
     const float* __restrict__ coef, int kp, int K, int nj, const float* __restrict__ rot,
     const float2* __restrict__ norm, const float* __restrict__ m, int s,
     const int* __restrict__ list, int n, float* __restrict__ comp, int first) {
-    static_assert(A % 2 == 0, "components in pairs");
-    constexpr int AP = (A + 3) & ~3;                  // rows of whole float4
+    static_assert(A % 4 == 0, "coefficients are copied and read four at a time");
     constexpr int J = 16;                             // nodes per step
-    __shared__ __align__(16) float cs[J][AP];
-    __shared__ float2 ns[J];
+    __shared__ __align__(16) float cs[2][J][A];
+    __shared__ __align__(16) float raw[2][J][V * kFold2Threads];
+    __shared__ __align__(8) float2 ns[2][J];
     const int a0 = blockIdx.y * A;
     const int t = threadIdx.x;
     const int s3 = s * s * s;
@@ -477,44 +489,59 @@ __global__ void __launch_bounds__(kFold2Threads) fold_list_kernel(
     for (int k = 0; k < V; ++k)
 #pragma unroll
         for (int a = 0; a < A / 2; ++a) acc[k][a] = f2(0.f, 0.f);
-    float raw[V][J];
-    auto fetch = [&](int jb) {
+    // nodes jb .. jb + J - 1 (zeros past the last, and for threads past the list)
+    auto stage = [&](int jb, int buf) {
 #pragma unroll
         for (int jj = 0; jj < J; ++jj)
 #pragma unroll
-            for (int k = 0; k < V; ++k)
-                raw[k][jj] = jb + jj < nj && at[k] >= 0 ? __ldg(rot + (size_t)(jb + jj) * n + at[k]) : 0.f;
-    };
-    for (int jb = 0; jb < nj; jb += J) {
-        fetch(jb);
-        __syncthreads();
-        for (int e = t; e < J * A; e += kFold2Threads) {
-            const int jj = e / A, a = e - jj * A;
-            cs[jj][a] = jb + jj < nj ? __ldg(coef + (size_t)(jb + jj) * kp + a0 + a) : 0.f;
+            for (int k = 0; k < V; ++k) {
+                float* d = &raw[buf][jj][k * kFold2Threads + t];
+                if (jb + jj < nj && at[k] >= 0) copy_async(d, rot + (size_t)(jb + jj) * n + at[k], 4);
+                else *d = 0.f;
+            }
+        for (int e = t; e < J * (A / 4); e += kFold2Threads) {
+            const int jj = e / (A / 4), q = e - jj * (A / 4);
+            float4* d = reinterpret_cast<float4*>(&cs[buf][jj][0]) + q;
+            if (jb + jj < nj) copy_async(d, coef + (size_t)(jb + jj) * kp + a0 + 4 * q, 16);
+            else *d = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        if (t < J) ns[t] = jb + t < nj ? norm[jb + t] : make_float2(0.f, 0.f);
+        if (t < J) {
+            if (jb + t < nj) copy_async(&ns[buf][t], norm + jb + t, 8);
+            else ns[buf][t] = make_float2(0.f, 0.f);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    stage(0, 0);
+    int buf = 0;
+    for (int jb = 0; jb < nj; jb += J, buf ^= 1) {
+        if (jb + J < nj) {
+            stage(jb + J, buf ^ 1);
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        }
         __syncthreads();
 #pragma unroll
         for (int jj = 0; jj < J; ++jj) {
-            const float2 nm = ns[jj];
+            const float2 nm = ns[buf][jj];
             F2 r[V];
 #pragma unroll
             for (int k = 0; k < V; ++k) {
-                const float x = mv[k] * (raw[k][jj] - nm.x) * nm.y;
+                const float x = mv[k] * (raw[buf][jj][k * kFold2Threads + t] - nm.x) * nm.y;
                 r[k] = f2(x, x);
             }
-            const float4* c4 = reinterpret_cast<const float4*>(&cs[jj][0]);
+            const float4* c4 = reinterpret_cast<const float4*>(&cs[buf][jj][0]);
 #pragma unroll
-            for (int q = 0; q < AP / 4; ++q) {
+            for (int q = 0; q < A / 4; ++q) {
                 const float4 c = c4[q];
 #pragma unroll
                 for (int k = 0; k < V; ++k) {
                     acc[k][2 * q] = f2_fma(f2(c.x, c.y), r[k], acc[k][2 * q]);
-                    if (4 * q + 2 < A) acc[k][2 * q + 1 < A / 2 ? 2 * q + 1 : 0] =
-                        f2_fma(f2(c.z, c.w), r[k], acc[k][2 * q + 1 < A / 2 ? 2 * q + 1 : 0]);
+                    acc[k][2 * q + 1] = f2_fma(f2(c.z, c.w), r[k], acc[k][2 * q + 1]);
                 }
             }
         }
+        __syncthreads();                              // the buffer takes the next copies
     }
 #pragma unroll
     for (int k = 0; k < V; ++k) {
@@ -582,11 +609,12 @@ int list_blocks(int s) {
     return (b * b * z * 32 + kListThreads - 1) / kListThreads;
 }
 // components per pass of fold_list_kernel, and the coefficient rows' length:
-// 42 (two passes at order 6, one at order 4) with two voxels per thread where
-// that still gives every SM two CTAs, else 12 with one voxel
-constexpr int kFoldWide = 42, kFoldNarrow = 12;
-int fold_row(int K) {
-    const int wide = (K + kFoldWide - 1) / kFoldWide * kFoldWide;
+// one pass of 36 at order 4, 44 at orders 6 and 8, with two voxels per thread
+// where that still gives every SM two CTAs, else 12 with one voxel
+constexpr int kFoldNarrow = 12;
+constexpr int fold_wide(int K) { return K <= 36 ? 36 : 44; }
+constexpr int fold_row(int K) {
+    const int wide = (K + fold_wide(K) - 1) / fold_wide(K) * fold_wide(K);
     const int narrow = (K + kFoldNarrow - 1) / kFoldNarrow * kFoldNarrow;
     return wide > narrow ? wide : narrow;
 }
@@ -595,16 +623,17 @@ template <int N>
 ttm_status fold_list_n(const TemplateBuild& b, const float* quats, const float* weights, int n_rot,
                        int j0, int nj, float* comp, bool first, cudaStream_t st, long long* cnt) {
     constexpr int K = n_comp(N);
+    constexpr int A = fold_wide(K);
     const int kp = fold_row(K);
     coef_kernel<N><<<(nj + 127) / 128, 128, 0, st>>>(quats, weights, 1.0f / (float)n_rot, j0, nj, kp,
                                                      b.coef);
     TTM_TRY(after_launch(cnt));
-    const int wide = (K + kFoldWide - 1) / kFoldWide;
+    const int wide = (K + A - 1) / A;
     const int narrow = (K + kFoldNarrow - 1) / kFoldNarrow;
     const int per2 = 2 * kFold2Threads;
     if (K > kFoldNarrow && (b.n + per2 - 1) / per2 * wide >= 304) {
         const dim3 grid((b.n + per2 - 1) / per2, wide);
-        fold_list_kernel<kFoldWide, 2><<<grid, kFold2Threads, 0, st>>>(
+        fold_list_kernel<A, 2><<<grid, kFold2Threads, 0, st>>>(
             b.coef, kp, K, nj, b.rot, b.norm, b.mask, b.s, b.list, b.n, comp, first);
     } else {
         const dim3 grid((b.n + kFold2Threads - 1) / kFold2Threads, narrow);
@@ -617,12 +646,13 @@ ttm_status fold_list_n(const TemplateBuild& b, const float* quats, const float* 
 
 static_assert(sizeof(VoxelList) <= 64, "the prepass results sit in the workspace header");
 
-// The prepass: mask sum, voxel list and flags into the header at `head`; the
+// The prepass: voxel list and flags into the header at `head` (a binary mask's
+// sum is its number of voxels: no mask sum is formed, whose FP64 additions in one
+// CTA took 150 us at 64^3); the
 // list at the start of `area`, its CTA counts at the end of the area_floats.
 ttm_status launch_build_prepass(const float* t, const float* m, int s, void* head, float* area,
                                 size_t area_floats, cudaStream_t st, long long* cnt) {
     VoxelList* vl = reinterpret_cast<VoxelList*>(head);
-    TTM_TRY(launch_mask_sum(m, s, &vl->mask_sum, st, cnt));
     const int nb = list_blocks(s);
     int* counts = reinterpret_cast<int*>(area + area_floats - nb);
     list_count_kernel<<<nb, kListThreads, 0, st>>>(t, m, s, counts, vl);
@@ -636,11 +666,19 @@ bool build_prepass_fits(int s, size_t area_floats) {
     return area_floats >= (size_t)s * s * s + (size_t)list_blocks(s);
 }
 
+// The sum of a binary, finite mask from the prepass; false for another.
+bool build_mask_count(const void* head_host, double* mask_sum) {
+    const VoxelList& vl = *reinterpret_cast<const VoxelList*>(head_host);
+    if (vl.odd || vl.soft) return false;
+    *mask_sum = (double)vl.n;
+    return true;
+}
+
 // Splits the area behind the list: cells, norms, coefficients, rotated rows of
 // up to nj nodes.  False where they do not fit (a mask that fills its box, a
 // handful of nodes) or values are not finite: the build then takes every voxel.
-bool build_layout(const void* head_host, const float* m, int s, int n_order, int nj, float* area,
-                  size_t area_floats, TemplateBuild* out) {
+bool build_layout(const void* head_host, const float* m, double mask_sum, int s, int n_order, int nj,
+                  float* area, size_t area_floats, TemplateBuild* out) {
     const VoxelList& vl = *reinterpret_cast<const VoxelList*>(head_host);
     if (vl.odd || vl.n < 1) return false;
     const size_t side = (size_t)s + 3;
@@ -649,7 +687,7 @@ bool build_layout(const void* head_host, const float* m, int s, int n_order, int
                  coef = up((size_t)nj * fold_row(n_comp(n_order))), rot = (size_t)nj * vl.n;
     if (list + cells + norm + coef + rot > area_floats) return false;
     out->s = s; out->n = vl.n; out->soft = vl.soft; out->mask = m;
-    out->mask_sum = vl.mask_sum;
+    out->mask_sum = mask_sum;
     out->list = reinterpret_cast<int*>(area);
     out->cells = area + list;
     out->norm = reinterpret_cast<float2*>(area + list + cells);
@@ -669,7 +707,7 @@ ttm_status launch_build_nodes(const TemplateBuild& b, int n_order, const float* 
                               const float* weights, int n_rot, int j0, int nj, float* comp,
                               int* d_bad, cudaStream_t st, long long* cnt) {
     // small masks: fewer warps to reduce per node
-    const int threads = b.n < 4096 ? 128 : kRotThreads;
+    const int threads = b.n < 4096 ? 128 : 256;
     rotate_list_kernel<<<nj, threads, 0, st>>>(reinterpret_cast<const float4*>(b.cells), b.mask, b.s,
                                                quats, j0, b.list, b.n, b.soft, b.rot, b.norm,
                                                b.mask_sum, d_bad);

@@ -170,6 +170,45 @@ ttm_status build_grid(ttm_plan_s* P) {
     return TTM_OK;
 }
 
+// The marching form of a small mask (MarchMask), or n_win = 0.
+MarchMask march_mask(const TemplateData& T, std::vector<int>& out) {
+    MarchMask m;
+    const int ndz = T.dz_max - T.dz_min + 1;
+    if (ndz > kMarchDz || T.dy_max - T.dy_min >= kMarchDz || T.x_max - T.x_min >= kMarchDz) return m;
+    std::vector<std::pair<int, int>> win;
+    for (const MaskRun& r : T.runs) {
+        const std::pair<int, int> w(r.x0, r.x1);
+        if (std::find(win.begin(), win.end(), w) == win.end()) win.push_back(w);
+    }
+    if ((int)win.size() > kMarchWin) return m;
+    std::sort(win.begin(), win.end(), [](const std::pair<int, int>& a, const std::pair<int, int>& b) {
+        return a.second - a.first != b.second - b.first ? a.second - a.first < b.second - b.first : a < b;
+    });
+    std::vector<std::vector<int>> cls;
+    for (int dz = T.dz_min; dz <= T.dz_max; ++dz) {
+        std::vector<int> runs;
+        for (const MaskRun& r : T.runs)
+            if (r.dz == dz)
+                runs.push_back((r.dy - T.dy_min) |
+                               (int)(std::find(win.begin(), win.end(), std::make_pair(r.x0, r.x1)) - win.begin()) << 8);
+        size_t c = std::find(cls.begin(), cls.end(), runs) - cls.begin();
+        if (c == cls.size()) cls.push_back(runs);
+        m.cls[dz - T.dz_min] = (int)c;
+    }
+    for (size_t c = 0; c < cls.size(); ++c) {
+        m.run0[c] = (int)out.size();
+        out.insert(out.end(), cls[c].begin(), cls[c].end());
+    }
+    m.n_cls = (int)cls.size();
+    m.run0[m.n_cls] = (int)out.size();
+    for (size_t k = 0; k < win.size(); ++k) {
+        m.x0[k] = win[k].first;
+        m.x1[k] = win[k].second;
+    }
+    m.n_win = (int)win.size();
+    return m;
+}
+
 // Mask -> x-runs and tap-major component table.
 ttm_status prepare_template(ttm_plan_s* P, TemplateData& T, const float* d_mask) {
     const int s = T.desc.s, c = T.desc.centre, K = T.desc.K;
@@ -242,6 +281,9 @@ ttm_status prepare_template(ttm_plan_s* P, TemplateData& T, const float* d_mask)
     TTM_TRY(dev_upload(&T.d_run_tap0, tap0));
     TTM_TRY(dev_upload(&T.d_dz_run0, dz0));
     TTM_TRY(dev_upload(&T.d_taps, taps));
+    std::vector<int> march_runs;
+    T.march = march_mask(T, march_runs);
+    TTM_TRY(dev_upload(&T.d_march_runs, march_runs));
     if (direct_tc_supported(K, ntap)) {
         // tensor-core direct path: FP16 component table and per-tap offsets
         std::vector<uint16_t> tab;
@@ -405,6 +447,7 @@ void free_plan(ttm_plan_s* P) {
         cudaFree(T.d_mask);
         cudaFree(T.d_run_tap0);
         cudaFree(T.d_dz_run0);
+        cudaFree(T.d_march_runs);
         cudaFree(T.d_taps);
         cudaFree(T.d_tc_tab);
         cudaFree(T.d_tap_dxyz);
@@ -1111,10 +1154,17 @@ ttm_status ttm_build_tensor_template(const float* d_template, const float* d_mas
     TTM_CUDA_TRY(cudaMemcpyAsync(head, ws, sizeof(head), cudaMemcpyDeviceToHost, st));
     TTM_CUDA_TRY(cudaStreamSynchronize(st));
     double msum = 0.0;
-    std::memcpy(&msum, head, sizeof(msum));
+    if (!prepass) {
+        std::memcpy(&msum, head, sizeof(msum));
+    } else if (!build_mask_count(head, &msum)) {
+        TTM_TRY(launch_mask_sum(d_mask, s, (double*)ws, st, &cnt));
+        TTM_CUDA_TRY(cudaMemcpyAsync(&msum, ws, sizeof(msum), cudaMemcpyDeviceToHost, st));
+        TTM_CUDA_TRY(cudaStreamSynchronize(st));
+    }
     if (!(msum > 0.0)) return TTM_ERR_INVALID_ARG;
     TemplateBuild tb;
-    const bool listed = prepass && build_layout(head, d_mask, s, n_order, nj, rot, area, &tb);
+    const bool listed = prepass && build_layout(head, d_mask, msum, s, n_order, nj, rot, area,
+                                             &tb);
     if (listed) {
         TTM_TRY(launch_build_cells(tb, d_template, st, &cnt));
         // voxels outside the mask

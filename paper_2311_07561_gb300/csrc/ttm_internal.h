@@ -13,6 +13,19 @@ struct MaskRun {
     int dy, dz, x0, x1;
 };
 
+// Small binary masks for the marching local statistics (k_stats.cu): the
+// distinct x-windows of the mask's runs, ordered so that each extends an
+// earlier one where it contains it, and the distinct planes as lists of runs
+// (dy - dy_min) | window << 8; mask plane dz belongs to class cls[dz - dz_min].
+constexpr int kMarchWin = 8, kMarchDz = 15;
+struct MarchMask {
+    int n_win = 0;                      // 0: the mask does not qualify
+    int x0[kMarchWin], x1[kMarchWin];
+    int n_cls = 0;
+    int run0[kMarchDz + 1];             // runs of class c: run0[c] .. run0[c + 1] - 1
+    int cls[kMarchDz];
+};
+
 // Plan-side image of one template.
 struct TemplateData {
     ttm_tt_desc desc{};
@@ -25,6 +38,8 @@ struct TemplateData {
     MaskRun* d_runs = nullptr;          // device copy of runs
     int* d_run_tap0 = nullptr;          // first tap index of every run
     int* d_dz_run0 = nullptr;           // first run of every dz plane (dz_max-dz_min+2)
+    MarchMask march;                    // small masks
+    int* d_march_runs = nullptr;
     float* d_taps = nullptr;            // n_taps x K component values, tap-major
     // tensor-core direct path (small masks): FP16 table of T / max|T| in the
     // kernel's layout, per-tap offsets (dx, dy, dz) packed, and max|T|
@@ -311,8 +326,9 @@ struct TemplateBuild {
 bool build_prepass_fits(int s, size_t area_floats);
 ttm_status launch_build_prepass(const float* t, const float* m, int s, void* head, float* area,
                                 size_t area_floats, cudaStream_t st, long long* cnt);
-bool build_layout(const void* head_host, const float* m, int s, int n_order, int nj, float* area,
-                  size_t area_floats, TemplateBuild* out);
+bool build_mask_count(const void* head_host, double* mask_sum);
+bool build_layout(const void* head_host, const float* m, double mask_sum, int s, int n_order, int nj,
+                  float* area, size_t area_floats, TemplateBuild* out);
 ttm_status launch_build_cells(const TemplateBuild& b, const float* t, cudaStream_t st, long long* cnt);
 ttm_status launch_build_nodes(const TemplateBuild& b, int n_order, const float* quats,
                               const float* weights, int n_rot, int j0, int nj, float* comp,
