@@ -888,6 +888,13 @@ cudaError_t run_cols_mul(const float2* spec, const TS* tspec, PS* prod, int Bz, 
 // single CTA per SM is left (960: scalar 421 us, packed 438; 1024: 432, 740)
 template <int L> constexpr bool rows_packed() { return (c2r_half<L>() || two_level<L>()) && L < 960; }
 
+// forward rows of a volume: the packed pass where the second step has at most
+// one item per thread (256: 108 -> 41 us for 256 x 250 x 230; 480: 203 -> 74)
+template <int L> constexpr bool rowsf_packed() {
+    if constexpr (r2c_half<L>()) return rowsf_ok<RowSplit<L / 2>::L1, RowSplit<L / 2>::L2>();
+    return false;
+}
+
 template <int L, typename PS, typename RT>
 cudaError_t run_rows_c2r(const PS* prod, int X, int Y, int Z, FftGeom g, RT* corr, int K,
                          const float2* tw, int* status, FftKeep keep, cudaStream_t st) {
@@ -955,6 +962,28 @@ template <int L>
 cudaError_t FftLen<L>::rows_r2c(const float* f, int X, int Y, int Z, FftGeom g, float2* spec,
                                 const float2* tw, int mode, double* moments, BoxIn box,
                                 cudaStream_t st) {
+    if constexpr (fftk::rowsf_packed<L>()) {
+        if (box.s == 0) {
+            constexpr int L1 = fftk::RowSplit<L / 2>::L1, L2 = fftk::RowSplit<L / 2>::L2;
+            constexpr int NR = 2 * fftk::rowp_pairs<L1, L2>();
+            constexpr size_t smem = fftk::rowsf_smem<L1, L2>();
+            auto kern = fftk::rowsf_t<L1, L2>;
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem);
+            if (e != cudaSuccess) return e;
+            const size_t nrows = (size_t)g.Yp * g.Zp;
+            unsigned grid = 0;
+            if ((e = fftk::persistent_grid(kern, smem, (nrows + NR - 1) / NR, &grid, fftk::kRowThreads)) !=
+                cudaSuccess)
+                return e;
+            if (grid == 0) return cudaSuccess;
+            // floats per copy: what the volume's address and its rows allow
+            const int vec = X % 4 == 0 && (uintptr_t)f % 16 == 0 ? 4
+                          : X % 2 == 0 && (uintptr_t)f % 8 == 0 ? 2 : 1;
+            kern<<<grid, fftk::kRowThreads, smem, st>>>(f, X, Y, Z, g, spec, tw, mode, moments, vec);
+            return cudaGetLastError();
+        }
+    }
     if constexpr (fftk::r2c_half<L>()) {
         constexpr int L1 = fftk::RowSplit<L / 2>::L1, L2 = fftk::RowSplit<L / 2>::L2;
         constexpr int NR = fftk::kTwoThreads / L1;

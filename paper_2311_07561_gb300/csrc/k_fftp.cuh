@@ -685,5 +685,162 @@ __global__ void __launch_bounds__(kRowThreads, (rowp_ctas<L1, L2, HALF, PS>())) 
     }
 }
 
+// ---- real x lines -> half-spectrum rows (rows_r2c_half_t, two rows a thread) ----
+// The rows of a tile are copied into shared memory (16, 8 or 4 bytes a copy, as
+// their alignment allows), the next tile's while this one goes through its
+// second step and the pairing; after the second step the transforms Z go back
+// to shared memory, where X[k] finds Z[k] and Z[M - k].
+template <int L1, int L2> constexpr bool rowsf_ok() { return rowp_pairs<L1, L2>() * L2 <= kRowThreads; }
+template <int L1, int L2> constexpr size_t rowsf_smem() {
+    constexpr int M = L1 * L2, NR = 2 * rowp_pairs<L1, L2>();
+    return (size_t)M * 16 + (size_t)rowp_pairs<L1, L2>() * L2 * (L1 + 1) * 16 + (size_t)NR * 2 * M * 4 +
+           (size_t)2 * NR * 8;
+}
+template <int L1, int L2> constexpr int rowsf_ctas() {
+    constexpr int by_regs = 65536 / (kRowThreads * ((c2_regs<L1, L2>() + 7) / 8 * 8));
+    constexpr int by_smem = (int)((size_t)227 * 1024 / (rowsf_smem<L1, L2>() + 1024));
+    return by_regs < by_smem ? by_regs : by_smem;
+}
+
+template <int L1, int L2>
+__global__ void __launch_bounds__(kRowThreads, (rowsf_ctas<L1, L2>())) rowsf_t(
+    const float* __restrict__ f, int X, int Y, int Z, FftGeom g, float2* __restrict__ out,
+    const float2* __restrict__ tw, int mode, double* __restrict__ moments, int vec) {
+    constexpr int M = L1 * L2, L = 2 * M;
+    constexpr int XP = spec_pitch(L);
+    constexpr int NPR = rowp_pairs<L1, L2>(), NR = 2 * NPR;
+    extern __shared__ __align__(16) unsigned char smp[];
+    float4* twm = reinterpret_cast<float4*>(smp);                 // W_M^j
+    float4* zx = twm + M;
+    float* st = reinterpret_cast<float*>(zx + NPR * L2 * (L1 + 1));
+    long long* rows = reinterpret_cast<long long*>(st + NR * L);  // inputs of two tiles in turn, -1: zero row
+    __shared__ double part[kRowThreads / 32];
+    __shared__ float mean_s;
+    const int t = threadIdx.x;
+    const size_t nrows = (size_t)g.Yp * g.Zp;
+    const size_t ntiles = (nrows + NR - 1) / NR;
+    auto list_rows = [&](size_t tile, long long* r) {
+        if (t >= NR) return;
+        const size_t q = tile * NR + t;
+        long long src = -1;
+        if (q < nrows) {
+            const uint32_t y = (uint32_t)(q % (size_t)g.Yp), z = (uint32_t)(q / (size_t)g.Yp);
+            if (y < (uint32_t)Y && z < (uint32_t)Z) src = (long long)(((size_t)z * Y + y) * X);
+        }
+        r[t] = src;
+    };
+    auto copy = [&](const long long* r) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(st);
+        const int per = X / vec;                                  // copies per row
+        for (int e = t; e < NR * per; e += kRowThreads) {
+            const int row = e / per, c = (e - row * per) * vec;
+            const long long src = r[row];
+            if (src < 0) continue;
+            const uint32_t d = dst + (uint32_t)(row * L + c) * 4;
+            if (vec == 4) cp_async16(d, f + src + c);
+            else if (vec == 2) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(f + src + c) : "memory");
+            else cp_async4(d, f + src + c);
+        }
+        cp_async_commit();
+    };
+    size_t tile = blockIdx.x;
+    if (tile >= ntiles) return;
+    if (t == 0) mean_s = mode ? (float)(moments[0] / ((double)X * Y * Z)) : 0.f;
+    list_rows(tile, rows);
+    for (int e = t; e < NR * L; e += kRowThreads) st[e] = 0.f;    // samples from X on stay zero
+    __syncthreads();
+    copy(rows);
+    for (int m = t; m < M; m += kRowThreads) {
+        const float2 w = __ldg(tw + 2 * m);
+        twm[m] = make_float4(w.x, w.x, w.y, w.y);
+    }
+    const float mean = mean_s;
+    float q4 = 0.f;                                               // mode 2: sum of (f - mean)^4
+    for (int cur = 0; tile < ntiles; tile += gridDim.x, cur ^= 1) {
+        const bool more = tile + gridDim.x < ntiles;
+        const long long* mine = rows + cur * NR;
+        cp_async_wait_all();
+        __syncthreads();                 // the rows in place, the exchange and the other list free
+        if (more) list_rows(tile + gridDim.x, rows + (cur ^ 1) * NR);
+#pragma unroll 1
+        for (int it = t; it < NPR * L1; it += kRowThreads) {
+            const int rp = it / L1, n1 = it % L1;
+            const bool ina = mine[2 * rp] >= 0, inb = mine[2 * rp + 1] >= 0;
+            const float* pa = st + (2 * rp) * L;
+            C2 v[L2];
+#pragma unroll
+            for (int n2 = 0; n2 < L2; ++n2) {
+                const int x = 2 * (n1 + L1 * n2);
+                float2 a = *reinterpret_cast<const float2*>(pa + x);
+                float2 b = *reinterpret_cast<const float2*>(pa + L + x);
+                a.x = ina && x < X ? a.x - mean : 0.f;
+                a.y = ina && x + 1 < X ? a.y - mean : 0.f;
+                b.x = inb && x < X ? b.x - mean : 0.f;
+                b.y = inb && x + 1 < X ? b.y - mean : 0.f;
+                if (mode == 2) {
+                    a.x *= a.x; a.y *= a.y; b.x *= b.x; b.y *= b.y;
+                    q4 = fmaf(a.x, a.x, fmaf(a.y, a.y, q4));
+                    q4 = fmaf(b.x, b.x, fmaf(b.y, b.y, q4));
+                }
+                v[n2] = C2{f2(a.x, b.x), f2(a.y, b.y)};
+            }
+            c2_dft<L2, -1>(v);
+#pragma unroll
+            for (int k2 = 0; k2 < L2; ++k2) {
+                if (k2 > 0) v[k2] = c2_mul_tab<-1>(v[k2], twm + n1 * k2);
+                zx[(rp * L2 + k2) * (L1 + 1) + n1] = make_float4(f2_get(v[k2].re, 0), f2_get(v[k2].re, 1),
+                                                                f2_get(v[k2].im, 0), f2_get(v[k2].im, 1));
+            }
+        }
+        __syncthreads();
+        if (more) copy(rows + (cur ^ 1) * NR);
+        const int rp = t / L2, k2 = t % L2;
+        C2 u[L1];
+        if (rp < NPR) {
+#pragma unroll
+            for (int m = 0; m < L1; ++m) {
+                const float4 q = zx[(rp * L2 + k2) * (L1 + 1) + m];
+                u[m] = C2{f2(q.x, q.y), f2(q.z, q.w)};
+            }
+            c2_dft<L1, -1>(u);
+        }
+        __syncthreads();                 // the exchange takes Z
+        if (rp < NPR) {
+#pragma unroll
+            for (int k1 = 0; k1 < L1; ++k1)
+                zx[rp * M + k2 + L2 * k1] = make_float4(f2_get(u[k1].re, 0), f2_get(u[k1].re, 1),
+                                                        f2_get(u[k1].im, 0), f2_get(u[k1].im, 1));
+        }
+        __syncthreads();
+        for (int e = t; e < NPR * (M + 1); e += kRowThreads) {
+            const int p = e / (M + 1), k = e - p * (M + 1);
+            const size_t q = tile * NR + 2 * p;
+            if (q >= nrows) continue;
+            const float4 za = zx[p * M + (k == M ? 0 : k)], zb = zx[p * M + (k == 0 ? 0 : M - k)];
+            const C2 a{f2(za.x, za.y), f2(za.z, za.w)}, b{f2(zb.x, zb.y), f2(zb.z, zb.w)};
+            const float2 w = __ldg(tw + k);
+            const F2 h = dup2(0.5f);
+            // b stands for conj Z[M - k]
+            const C2 s{f2_mul(h, f2_add(a.re, b.re)), f2_mul(h, f2_sub(a.im, b.im))};
+            const C2 d = c2_mul<false, false>(C2{f2_mul(h, f2_sub(a.re, b.re)), f2_mul(h, f2_add(a.im, b.im))},
+                                              dup2(w.x), dup2(w.y), dup2(-w.y));
+            const F2 re = f2_add(s.re, d.im), im = f2_sub(s.im, d.re);     // s - i d
+            out[q * XP + k] = make_float2(f2_get(re, 0), f2_get(im, 0));
+            if (q + 1 < nrows) out[(q + 1) * XP + k] = make_float2(f2_get(re, 1), f2_get(im, 1));
+        }
+    }
+    if (mode == 2) {
+        double d = q4;
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+        if ((t & 31) == 0) part[t >> 5] = d;
+        __syncthreads();
+        if (t == 0) {
+            double s4 = 0.0;
+            for (int k = 0; k < kRowThreads / 32; ++k) s4 += part[k];
+            if (s4 != 0.0) atomicAdd(moments + 2, s4);
+        }
+    }
+}
+
 }  // namespace fftk
 }  // namespace ttm

@@ -422,12 +422,13 @@ ttm_status launch_local_stats(const float* f, int X, int Y, int Z, const Templat
     if (T.march.n_win > 0 && box.count() > 0) {
         // every output's planes lie in the volume (a mask reaches at most its
         // box).  Planes per CTA: fewer cost more halo planes, more leave SMs
-        // idle; enough CTAs for two per SM, at least 8 planes
+        // idle; at most two CTAs per SM (FP64 sets the pace, so a third on some
+        // SMs is half the time again), at least 8 planes
         MarchArgs m;
         m.s = a; m.m = T.march; m.runs = T.d_march_runs;
         m.x0 = box.x0; m.y0 = box.y0; m.z0 = box.z0; m.z1 = box.z0 + (int)box.nz - 1;
         const int gx = ((int)box.nx + kMarchX - 1) / kMarchX, gy = ((int)box.ny + kMarchY - 1) / kMarchY;
-        const int want = (304 + gx * gy - 1) / (gx * gy);
+        const int want = 304 / (gx * gy) > 1 ? 304 / (gx * gy) : 1;
         int nzc = ((int)box.nz + want - 1) / want;
         nzc = nzc < 8 ? 8 : nzc > 64 ? 64 : nzc;
         m.nzc = nzc;

@@ -318,6 +318,9 @@ __device__ __forceinline__ float two_sum(float a, float b, float& e) {
     return s;
 }
 
+// row length of the rotated samples: rows start on 16 bytes
+__host__ __device__ constexpr size_t rot_pitch(int n) { return ((size_t)n + 3) & ~(size_t)3; }
+
 // One CTA per node: raw samples of the listed voxels, and the node's offset
 // and scale.  FP64 runs at 1/64 of the FP32 rate here, so the sums of four
 // samples (and of their exact squares) are formed in FP32 without error, sum
@@ -337,7 +340,7 @@ __global__ void __launch_bounds__(256, 5) rotate_list_kernel(
     const float c = (float)(s / 2);
     const int side = s + 3, plane = side * side;
     const float top = (float)s;
-    float* o = out + (size_t)blockIdx.x * n;
+    float* o = out + (size_t)blockIdx.x * rot_pitch(n);
     double t1 = 0.0, t2 = 0.0;
     float e1 = 0.f, e2 = 0.f;
     for (int i0 = threadIdx.x; i0 < n; i0 += 4 * blockDim.x) {
@@ -446,14 +449,17 @@ __global__ void __launch_bounds__(128) coef_kernel(const float* __restrict__ qua
 // T_alpha(u) over the listed voxels, A components (blockIdx.y) and V voxels per
 // thread: a coefficient pair read from shared memory (a broadcast) feeds V
 // packed FMAs of two components each.  The samples, coefficients and norms of
-// the next 16 nodes are copied into shared memory while this step's are folded
+// the next nodes are copied into shared memory while this step's are folded
 // (loading them into registers at the step's start left the FMA pipe idle two
 // thirds of the time: 30.5 ms at 64^3, order 6, 20000 rotations).  Bound by the
-// FMA pipe (packed: 116 FMAs a clock and SM).  A component's sum runs over the
+// shared-memory reads: 16 bytes for every lane take four clocks of the SM even
+// when they are one broadcast, so a coefficient quad has to feed four voxels (8
+// packed FMAs, four clocks of the FMA pipes).  A component's sum runs over the
 // nodes in order, as in fold_kernel.
 constexpr int kFold2Threads = 128;
 
-template <int A> constexpr int fold_ctas() { return A > 12 ? 3 : 6; }
+// V = 4: a thread's voxels are neighbours, copied and read as one float4
+template <int A, int V> constexpr int fold_ctas() { return V == 4 ? (A > 28 ? 2 : 3) : 6; }
 
 __device__ __forceinline__ void copy_async(void* dst, const void* src, int bytes) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
@@ -463,12 +469,12 @@ __device__ __forceinline__ void copy_async(void* dst, const void* src, int bytes
 }
 
 template <int A, int V>
-__global__ void __launch_bounds__(kFold2Threads, fold_ctas<A>()) fold_list_kernel(
+__global__ void __launch_bounds__(kFold2Threads, (fold_ctas<A, V>())) fold_list_kernel(
     const float* __restrict__ coef, int kp, int K, int nj, const float* __restrict__ rot,
     const float2* __restrict__ norm, const float* __restrict__ m, int s,
     const int* __restrict__ list, int n, float* __restrict__ comp, int first) {
     static_assert(A % 4 == 0, "coefficients are copied and read four at a time");
-    constexpr int J = 16;                             // nodes per step
+    constexpr int J = V == 4 ? 8 : 16;                // nodes per step
     __shared__ __align__(16) float cs[2][J][A];
     __shared__ __align__(16) float raw[2][J][V * kFold2Threads];
     __shared__ __align__(8) float2 ns[2][J];
@@ -479,7 +485,7 @@ __global__ void __launch_bounds__(kFold2Threads, fold_ctas<A>()) fold_list_kerne
     float mv[V];
 #pragma unroll
     for (int k = 0; k < V; ++k) {
-        const int i = (blockIdx.x * V + k) * kFold2Threads + t;
+        const int i = (blockIdx.x * kFold2Threads + t) * V + k;
         at[k] = i < n ? i : -1;
         vox[k] = at[k] >= 0 ? unpack_voxel(__ldg(list + i), s) : 0;
         mv[k] = at[k] >= 0 ? __ldg(m + vox[k]) : 0.f;
@@ -489,16 +495,18 @@ __global__ void __launch_bounds__(kFold2Threads, fold_ctas<A>()) fold_list_kerne
     for (int k = 0; k < V; ++k)
 #pragma unroll
         for (int a = 0; a < A / 2; ++a) acc[k][a] = f2(0.f, 0.f);
-    // nodes jb .. jb + J - 1 (zeros past the last, and for threads past the list)
+    const size_t pitch = rot_pitch(n);
+    // nodes jb .. jb + J - 1 (zeros past the last, and for threads past the
+    // list; a row's padding is copied, never used)
     auto stage = [&](int jb, int buf) {
 #pragma unroll
-        for (int jj = 0; jj < J; ++jj)
+        for (int jj = 0; jj < J; ++jj) {
+            float* d = &raw[buf][jj][V * t];
+            if (jb + jj < nj && at[0] >= 0) copy_async(d, rot + (jb + jj) * pitch + at[0], 4 * V);
+            else
 #pragma unroll
-            for (int k = 0; k < V; ++k) {
-                float* d = &raw[buf][jj][k * kFold2Threads + t];
-                if (jb + jj < nj && at[k] >= 0) copy_async(d, rot + (size_t)(jb + jj) * n + at[k], 4);
-                else *d = 0.f;
-            }
+                for (int k = 0; k < V; ++k) d[k] = 0.f;
+        }
         for (int e = t; e < J * (A / 4); e += kFold2Threads) {
             const int jj = e / (A / 4), q = e - jj * (A / 4);
             float4* d = reinterpret_cast<float4*>(&cs[buf][jj][0]) + q;
@@ -524,10 +532,18 @@ __global__ void __launch_bounds__(kFold2Threads, fold_ctas<A>()) fold_list_kerne
 #pragma unroll
         for (int jj = 0; jj < J; ++jj) {
             const float2 nm = ns[buf][jj];
+            float rw[V];
+            if constexpr (V == 4) {
+                const float4 q = *reinterpret_cast<const float4*>(&raw[buf][jj][V * t]);
+                rw[0] = q.x; rw[1] = q.y; rw[2] = q.z; rw[3] = q.w;
+            } else {
+#pragma unroll
+                for (int k = 0; k < V; ++k) rw[k] = raw[buf][jj][V * t + k];
+            }
             F2 r[V];
 #pragma unroll
             for (int k = 0; k < V; ++k) {
-                const float x = mv[k] * (raw[buf][jj][k * kFold2Threads + t] - nm.x) * nm.y;
+                const float x = mv[k] * (rw[k] - nm.x) * nm.y;
                 r[k] = f2(x, x);
             }
             const float4* c4 = reinterpret_cast<const float4*>(&cs[buf][jj][0]);
@@ -609,10 +625,11 @@ int list_blocks(int s) {
     return (b * b * z * 32 + kListThreads - 1) / kListThreads;
 }
 // components per pass of fold_list_kernel, and the coefficient rows' length:
-// one pass of 36 at order 4, 44 at orders 6 and 8, with two voxels per thread
-// where that still gives every SM two CTAs, else 12 with one voxel
+// one pass of 36 at order 4, three of 28 at order 6 (six at order 8) with four
+// voxels per thread where that gives every SM two CTAs, else 12 with two, else
+// 12 with one
 constexpr int kFoldNarrow = 12;
-constexpr int fold_wide(int K) { return K <= 36 ? 36 : 44; }
+constexpr int fold_wide(int K) { return K <= 36 ? 36 : 28; }
 constexpr int fold_row(int K) {
     const int wide = (K + fold_wide(K) - 1) / fold_wide(K) * fold_wide(K);
     const int narrow = (K + kFoldNarrow - 1) / kFoldNarrow * kFoldNarrow;
@@ -630,14 +647,15 @@ ttm_status fold_list_n(const TemplateBuild& b, const float* quats, const float* 
     TTM_TRY(after_launch(cnt));
     const int wide = (K + A - 1) / A;
     const int narrow = (K + kFoldNarrow - 1) / kFoldNarrow;
-    const int per2 = 2 * kFold2Threads;
-    if (K > kFoldNarrow && (b.n + per2 - 1) / per2 * wide >= 304) {
-        const dim3 grid((b.n + per2 - 1) / per2, wide);
-        fold_list_kernel<A, 2><<<grid, kFold2Threads, 0, st>>>(
+    auto blocks = [&](int v) { return (b.n + v * kFold2Threads - 1) / (v * kFold2Threads); };
+    if (K > kFoldNarrow && blocks(4) * wide >= 304) {
+        fold_list_kernel<A, 4><<<dim3(blocks(4), wide), kFold2Threads, 0, st>>>(
+            b.coef, kp, K, nj, b.rot, b.norm, b.mask, b.s, b.list, b.n, comp, first);
+    } else if (blocks(2) * narrow >= 152) {
+        fold_list_kernel<kFoldNarrow, 2><<<dim3(blocks(2), narrow), kFold2Threads, 0, st>>>(
             b.coef, kp, K, nj, b.rot, b.norm, b.mask, b.s, b.list, b.n, comp, first);
     } else {
-        const dim3 grid((b.n + kFold2Threads - 1) / kFold2Threads, narrow);
-        fold_list_kernel<kFoldNarrow, 1><<<grid, kFold2Threads, 0, st>>>(
+        fold_list_kernel<kFoldNarrow, 1><<<dim3(blocks(1), narrow), kFold2Threads, 0, st>>>(
             b.coef, kp, K, nj, b.rot, b.norm, b.mask, b.s, b.list, b.n, comp, first);
     }
     return after_launch(cnt);
@@ -684,7 +702,7 @@ bool build_layout(const void* head_host, const float* m, double mask_sum, int s,
     const size_t side = (size_t)s + 3;
     auto up = [](size_t v) { return (v + 63) & ~(size_t)63; };
     const size_t list = up((size_t)vl.n), cells = up(4 * side * side * (side + 1)), norm = up(2 * (size_t)nj),
-                 coef = up((size_t)nj * fold_row(n_comp(n_order))), rot = (size_t)nj * vl.n;
+                 coef = up((size_t)nj * fold_row(n_comp(n_order))), rot = (size_t)nj * rot_pitch(vl.n);
     if (list + cells + norm + coef + rot > area_floats) return false;
     out->s = s; out->n = vl.n; out->soft = vl.soft; out->mask = m;
     out->mask_sum = mask_sum;
