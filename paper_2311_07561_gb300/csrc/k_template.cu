@@ -325,7 +325,7 @@ __host__ __device__ constexpr size_t rot_pitch(int n) { return ((size_t)n + 3) &
 // and scale.  FP64 runs at 1/64 of the FP32 rate here, so the sums of four
 // samples (and of their exact squares) are formed in FP32 without error, sum
 // and remainder apart, and one FP64 addition takes the sum.
-__global__ void __launch_bounds__(256, 5) rotate_list_kernel(
+__global__ void __launch_bounds__(640, 2) rotate_list_kernel(
     const float4* __restrict__ cells, const float* __restrict__ m, int s,
     const float* __restrict__ quats, int j0, const int* __restrict__ list, int n, int soft,
     float* __restrict__ out, float2* __restrict__ norm, double mask_sum, int* bad) {
@@ -724,8 +724,12 @@ ttm_status launch_build_cells(const TemplateBuild& b, const float* t, cudaStream
 ttm_status launch_build_nodes(const TemplateBuild& b, int n_order, const float* quats,
                               const float* weights, int n_rot, int j0, int nj, float* comp,
                               int* d_bad, cudaStream_t st, long long* cnt) {
-    // small masks: fewer warps to reduce per node
-    const int threads = b.n < 4096 ? 128 : 256;
+    // small masks: fewer warps to reduce per node; few nodes (the 304 that a
+    // large mask's samples leave room for): two CTAs hold all the threads an SM
+    // takes at 48 registers (64^3 box, order 6, 20000 nodes: 40.9 -> 28.9 ms the
+    // build, against 256 threads); many nodes: 256 (32^3 box, 1024 nodes a
+    // chunk: 963 us of samples, 1061 with 512)
+    const int threads = b.n < 4096 ? 128 : nj <= 4 * 152 ? 640 : 256;
     rotate_list_kernel<<<nj, threads, 0, st>>>(reinterpret_cast<const float4*>(b.cells), b.mask, b.s,
                                                quats, j0, b.list, b.n, b.soft, b.rot, b.norm,
                                                b.mask_sum, d_bad);
