@@ -346,15 +346,18 @@ __device__ void refine(const float (&C)[Geo<N>::K4], float sigma, int newton, fl
     lam_out = la;
 }
 
-// ---- two candidates at a time (orders 2 and 4) -----------------------------
+// ---- two candidates at a time (orders 2, 4 and 6) --------------------------
 // The refinement is bound by the FMA pipe's register reads: scalar FMAs with
 // three different registers each ran at 78-86 lanes a clock and SM, packed
 // ones (fma.rn.f32x2, two FMAs per instruction) at 108.  So two candidates of
-// a voxel go through the evaluations together, one in each half of a register
-// pair; the components, which both share, are kept as pairs of equal halves
-// (2 K registers: orders 2 and 4 only, at order 6 they do not fit).  Every
-// half carries the operations of the scalar code in its order, so the results
-// are the same bits.
+// a voxel go through the evaluations and the Newton solves together, one in
+// each half of a register pair; the components, which both share, are kept as
+// pairs of equal halves (2 K registers: 168 at order 6, which leaves two CTAs
+// per SM and still gains; the 330 of order 8 do not fit).  Every half carries
+// the operations of the scalar code in its order, so the results are the same
+// bits.  Whole runs, evaluations packed -> solves too: order 4 at 512 x 512 x
+// 256, 29.8 -> 28.4 ms; order 6 at 928 x 464 x 232, all scalar before, 49.7 ->
+// 47.6 ms.
 template <int M>
 struct Monomials2 {
     F2 v[n_comp(M) > 0 ? n_comp(M) : 1];
@@ -424,103 +427,151 @@ __device__ __forceinline__ void eval2_at(const F2 (&C)[Geo<N>::K], const F2 (&x)
     lam = f2_dot(g, x);
 }
 
-// the next power step's point from (x, g): normalise(g + sigma x)
-static __device__ __forceinline__ void power_point(const float (&g)[4], float sigma, const float (&x)[4],
-                                                   float (&out)[4]) {
+// normalise4 for two points
+static __device__ __forceinline__ void normalise2(F2 (&x)[4]) {
+    const F2 n2 = f2_dot(x, x);
+    const F2 inv = f2(rsqrtf(f2_get(n2, 0)), rsqrtf(f2_get(n2, 1)));
 #pragma unroll
-    for (int i = 0; i < 4; ++i) out[i] = g[i] + sigma * x[i];
-    normalise4(out);
+    for (int i = 0; i < 4; ++i) x[i] = f2_mul(x[i], inv);
 }
 
 // power_steps for two candidates
 template <int N>
-__device__ __forceinline__ void power_steps2(const F2 (&C)[Geo<N>::K], float sigma, float (&xa)[4],
-                                             float (&xb)[4], float& la, float& lb, bool want_lam) {
-    F2 x[4], g[4], lam;
+__device__ __forceinline__ void power_steps2(const F2 (&C)[Geo<N>::K], float sigma, F2 (&x)[4],
+                                             F2& lam, bool want_lam) {
+    const F2 sig = f2(sigma, sigma);
+    F2 g[4];
 #pragma unroll 1
     for (int s = 0; s < 3; ++s) {
         if (s == 2 && !want_lam) break;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = f2(xa[i], xb[i]);
         grad2_at<N>(C, x, g, lam);
         if (s == 2) break;
-        float ga[4], gb[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            ga[i] = f2_get(g[i], 0);
-            gb[i] = f2_get(g[i], 1);
-        }
-        power_point(ga, sigma, xa, xa);
-        power_point(gb, sigma, xb, xb);
+        for (int i = 0; i < 4; ++i) x[i] = f2_fma(sig, x[i], g[i]);
+        normalise2(x);
     }
-    la = f2_get(lam, 0);
-    lb = f2_get(lam, 1);
 }
 
-// one point's state through refine: the last accepted point, its gradient and
-// value, and the trial
-struct RefineState {
-    float xa[4], ga[4], xt[4], la;
-    bool trial_newton;
-};
-
-// what refine does with the evaluation (h, g, lam) of the trial
+// newton_dir for two points: h = the entries of H, ok = each half's success.
+// A half whose factorisation breaks down leaves values that nobody reads.
 template <int N>
-__device__ __forceinline__ void refine_step(RefineState& r, const float (&h)[10],
-                                            const float (&g)[4], float lam, float sigma, float eps,
-                                            bool last) {
-    if (r.trial_newton && lam < r.la - eps) {
-        if (last) return;
-        power_point(r.ga, sigma, r.xa, r.xt);
-        r.trial_newton = false;
-        return;
-    }
+__device__ __forceinline__ void newton_dir2(const F2 (&h)[10], const F2 (&g)[4], const F2 (&x)[4],
+                                            F2 lam, float sig, F2 (&eta)[4], bool (&ok)[2]) {
+    const F2 minus = f2(-1.f, -1.f), nl = f2_mul(lam, minus);
+    const F2 order = f2((float)(N - 1), (float)(N - 1));
+    F2 B[4][4];
+    int p = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = i; j < 4; ++j, ++p) {
+            B[i][j] = i == j ? f2_fma(order, h[p], nl) : f2_mul(order, h[p]);
+            B[j][i] = B[i][j];
+        }
+    F2 Bx[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) Bx[i] = f2_dot(B[i], x);
+    const F2 cxx = f2_sub(f2_dot(x, Bx), f2(sig, sig));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) Bx[i] = f2_mul(Bx[i], minus);
+    // nA = -A and nL = -L: the same factorisation with every sign turned, as
+    // packed operations take no negated operand
+    F2 nA[4][4], nL[4][4], inv[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        r.xa[i] = r.xt[i];
-        r.ga[i] = g[i];
-    }
-    r.la = lam;
-    if (last) return;
-    float H[4][4], eta[4];
-    unpack(h, H);
-    if (newton_dir<N>(H, r.ga, r.xa, r.la, sigma, eta)) {
-        const float en2 = eta[0] * eta[0] + eta[1] * eta[1] + eta[2] * eta[2] + eta[3] * eta[3];
-        const float clip = en2 > 0.0625f ? 0.25f * rsqrtf(en2) : 1.f;
+        const F2 cx = f2_mul(cxx, x[i]);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) r.xt[i] = r.xa[i] + clip * eta[i];
-        r.trial_newton = true;
-        normalise4(r.xt);
-    } else {
-        power_point(r.ga, sigma, r.xa, r.xt);
-        r.trial_newton = false;
+        for (int j = 0; j <= i; ++j)
+            nA[i][j] = f2_fma(cx, x[j], f2_fma(x[i], Bx[j], f2_fma(Bx[i], x[j], B[i][j])));
+    }
+    const float tiny = 1e-9f * sig;
+    ok[0] = ok[1] = true;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        F2 d = nA[j][j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) d = f2_fma(nL[j][k], nL[j][k], d);
+        const float da = -f2_get(d, 0), db = -f2_get(d, 1);
+        ok[0] = ok[0] && da > tiny;
+        ok[1] = ok[1] && db > tiny;
+        inv[j] = f2(rsqrtf(da), rsqrtf(db));
+#pragma unroll
+        for (int i = j + 1; i < 4; ++i) {
+            F2 v = nA[i][j];
+#pragma unroll
+            for (int k = 0; k < j; ++k) v = f2_fma(nL[i][k], nL[j][k], v);
+            nL[i][j] = f2_mul(v, inv[j]);
+        }
+    }
+    F2 y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        F2 v = f2_fma(nl, x[i], g[i]);
+#pragma unroll
+        for (int k = 0; k < i; ++k) v = f2_fma(nL[i][k], y[k], v);
+        y[i] = f2_mul(v, inv[i]);
+    }
+#pragma unroll
+    for (int i = 3; i >= 0; --i) {
+        F2 v = y[i];
+#pragma unroll
+        for (int k = i + 1; k < 4; ++k) v = f2_fma(nL[k][i], eta[k], v);
+        eta[i] = f2_mul(v, inv[i]);
     }
 }
 
-// refine for two points
+static __device__ __forceinline__ F2 f2_pick(bool a, bool b, F2 yes, F2 no) {
+    return f2(a ? f2_get(yes, 0) : f2_get(no, 0), b ? f2_get(yes, 1) : f2_get(no, 1));
+}
+
+// refine for two points: from xt to the last accepted points xa and their
+// values.  Both halves form the Newton point; a half that goes by a power step
+// (a rejected trial, or no direction) takes g + sigma x of its accepted point
+// in its place before the common normalisation.
 template <int N>
 __device__ __forceinline__ void refine2(const F2 (&C)[Geo<N>::K], float sigma, int newton,
-                                        RefineState& a, RefineState& b) {
+                                        F2 (&xt)[4], F2 (&xa)[4], float& la, float& lb) {
     const float eps = 1e-6f * sigma;
+    const F2 sig = f2(sigma, sigma);
     const int iters = 1 + newton;
+    F2 ga[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        xa[i] = xt[i];
+        ga[i] = f2(0.f, 0.f);
+    }
+    la = lb = -INFINITY;
+    bool ta = false, tb = false;   // the trial is a Newton point
 #pragma unroll 1
     for (int it = 0; it < iters; ++it) {
         const bool last = it + 1 == iters;
-        F2 x[4], h[10], g[4], lam;
+        F2 h[10], g[4], lam;
+        // the last trial needs only phi (see refine)
+        if (N >= 6 && last && it > 0) grad2_at<N>(C, xt, g, lam);
+        else eval2_at<N>(C, xt, h, g, lam);
+        const float va = f2_get(lam, 0), vb = f2_get(lam, 1);
+        const bool keep_a = !(ta && va < la - eps), keep_b = !(tb && vb < lb - eps);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = f2(a.xt[i], b.xt[i]);
-        eval2_at<N>(C, x, h, g, lam);
-        float hs[10], gs[4];
+        for (int i = 0; i < 4; ++i) {
+            xa[i] = f2_pick(keep_a, keep_b, xt[i], xa[i]);
+            ga[i] = f2_pick(keep_a, keep_b, g[i], ga[i]);
+        }
+        la = keep_a ? va : la;
+        lb = keep_b ? vb : lb;
+        if (last) break;
+        F2 eta[4];
+        bool ok[2];
+        newton_dir2<N>(h, g, xt, lam, sigma, eta, ok);
+        const F2 en2 = f2_dot(eta, eta);
+        const float ea = f2_get(en2, 0), eb = f2_get(en2, 1);
+        const F2 clip = f2(ea > 0.0625f ? 0.25f * rsqrtf(ea) : 1.f,
+                           eb > 0.0625f ? 0.25f * rsqrtf(eb) : 1.f);
+        ta = ok[0] && keep_a;
+        tb = ok[1] && keep_b;
 #pragma unroll
-        for (int p = 0; p < 10; ++p) hs[p] = f2_get(h[p], 0);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) gs[i] = f2_get(g[i], 0);
-        refine_step<N>(a, hs, gs, f2_get(lam, 0), sigma, eps, last);
-#pragma unroll
-        for (int p = 0; p < 10; ++p) hs[p] = f2_get(h[p], 1);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) gs[i] = f2_get(g[i], 1);
-        refine_step<N>(b, hs, gs, f2_get(lam, 1), sigma, eps, last);
+        for (int i = 0; i < 4; ++i)
+            xt[i] = f2_pick(ta, tb, f2_fma(clip, eta[i], xa[i]), f2_fma(sig, xa[i], ga[i]));
+        normalise2(xt);
     }
 }
 
@@ -542,9 +593,9 @@ static __device__ __forceinline__ void keep_point(float (&kl)[kRefine], float (&
     }
 }
 
-template <int N> constexpr bool kPairs = N <= 4;
+template <int N> constexpr bool kPairs = N <= 6;
 
-// Refinement of a voxel's candidates, two at a time (orders 2 and 4); the
+// Refinement of a voxel's candidates, two at a time (orders 2, 4 and 6); the
 // scalar loops of polish_kernel state the steps.
 template <int N>
 __device__ __forceinline__ void polish_pairs(const float (&Cs)[Geo<N>::K4], float score,
@@ -573,16 +624,17 @@ __device__ __forceinline__ void polish_pairs(const float (&Cs)[Geo<N>::K4], floa
         int ib = (int)(pair >> 16);
         const bool two = k + 1 < nc && ib != 0xFFFF;
         if (!two) ib = ia;
-        float xa[4], xb[4], la, lb;
+        F2 x[4], lam;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = f2(__ldg(a.gq + 4 * ia + i), __ldg(a.gq + 4 * ib + i));
+        power_steps2<N>(C, sigma, x, lam, rank);
+        const float la = rank ? f2_get(lam, 0) : -(float)k;
+        const float lb = rank ? f2_get(lam, 1) : -(float)(k + 1);
+        float xa[4], xb[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            xa[i] = __ldg(a.gq + 4 * ia + i);
-            xb[i] = __ldg(a.gq + 4 * ib + i);
-        }
-        power_steps2<N>(C, sigma, xa, xb, la, lb, rank);
-        if (!rank) {
-            la = -(float)k;
-            lb = -(float)(k + 1);
+            xa[i] = f2_get(x[i], 0);
+            xb[i] = f2_get(x[i], 1);
         }
         keep_point(kl, kx, la, xa);
         if (!two) break;
@@ -592,28 +644,24 @@ __device__ __forceinline__ void polish_pairs(const float (&Cs)[Geo<N>::K4], floa
     for (int s = 0; s < kRefine; s += 2) {
         if (s >= a.n_refine || !((s == 0 ? kl[0] : kl[2]) > -INFINITY)) break;
         const bool two = s + 1 < a.n_refine && (s == 0 ? kl[1] : kl[3]) > -INFINITY;
-        RefineState ra, rb;
+        F2 xt[4], xa[4];
+        float la, lb;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             // the kept points s and s + 1, picked with compile-time indices
-            ra.xt[i] = s == 0 ? kx[0][i] : kx[2][i];
-            rb.xt[i] = !two ? ra.xt[i] : (s == 0 ? kx[1][i] : kx[3][i]);
-            ra.xa[i] = ra.xt[i];
-            rb.xa[i] = rb.xt[i];
-            ra.ga[i] = rb.ga[i] = 0.f;
+            const float p = s == 0 ? kx[0][i] : kx[2][i];
+            xt[i] = f2(p, !two ? p : (s == 0 ? kx[1][i] : kx[3][i]));
         }
-        ra.la = rb.la = -INFINITY;
-        ra.trial_newton = rb.trial_newton = false;
-        refine2<N>(C, sigma, a.newton, ra, rb);
-        if (ra.la > best_l) {
-            best_l = ra.la;
+        refine2<N>(C, sigma, a.newton, xt, xa, la, lb);
+        if (la > best_l) {
+            best_l = la;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) best_q[i] = ra.xa[i];
+            for (int i = 0; i < 4; ++i) best_q[i] = f2_get(xa[i], 0);
         }
-        if (two && rb.la > best_l) {
-            best_l = rb.la;
+        if (two && lb > best_l) {
+            best_l = lb;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) best_q[i] = rb.xa[i];
+            for (int i = 0; i < 4; ++i) best_q[i] = f2_get(xa[i], 1);
         }
     }
     static_assert(kRefine == 4 && kMaxCand % 2 == 0, "points in pairs");
@@ -691,9 +739,10 @@ __global__ void __launch_bounds__(kRotThreads) search_simt_kernel(const __grid_c
 }
 
 // CTAs per SM the refinement's registers are sized for: four (128 registers)
-// in pairs, three (168) at order 6, whose K = 84 components fill more; at
-// order 8 (K = 165) the components alone take all there are
-template <int N> constexpr int polish_ctas() { return N <= 4 ? 4 : N == 6 ? 3 : 2; }
+// at orders 2 and 4; two from order 6 on, whose K = 84 components as pairs fill
+// 168 (three CTAs spill 250 bytes a thread) and whose K = 165 at order 8 take
+// all there are
+template <int N> constexpr int polish_ctas() { return N <= 4 ? 4 : 2; }
 
 // Refinement of the candidates and the outputs: lambda = the largest refined
 // phi, q its maximiser (canonical sign), C_alpha optionally.
