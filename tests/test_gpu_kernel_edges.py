@@ -1,0 +1,189 @@
+"""The kernels at the sizes where their tiles, lists and variants end: FFT
+passes of every long length, window statistics of small masks, template builds
+over listed voxels, the candidates of the rotation search, peak lists.
+
+Tolerances are those of the parity tests: 1e-4 on components, score and lambda
+(FP32), 5e-3 with bf16 storage, 1e-5 relative on w, 2e-5 of the largest
+component on templates; peaks exact.
+"""
+
+import numpy as np
+import pytest
+
+import synth
+from oracle import ttm_oracle as o
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-4
+BF16_TOL = 5e-3
+
+
+@pytest.fixture(scope="module")
+def ttm():
+    import os
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    import paper_2311_07561_gb300 as ttm
+    if not os.path.exists(ttm.LIB_PATH):
+        import __graft_entry__
+        __graft_entry__.build()
+    ttm.load_library()
+    return ttm
+
+
+def _cuda(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+
+
+def _maps(ttm, volume, comp, desc, mask, want_comp=False, **opts):
+    import torch
+    po = ttm.PlanOpts()
+    for k, v in opts.items():
+        setattr(po, k, v)
+    Z, Y, X = volume.shape
+    m = ttm.Matcher([(comp, desc, mask)], [((X, Y, Z), 0)], opts=po)
+    comps = [torch.empty((desc.K, Z, Y, X), dtype=torch.float32, device="cuda")] if want_comp else None
+    m.run([_cuda(volume)], components_out=comps)
+    torch.cuda.synchronize()
+    assert ttm.ttm_plan_device_status(m.plan, m.ws) == 0
+    out = dict(w=m.w[0].cpu().numpy(), score=m.score[0].cpu().numpy(),
+               quat=m.quat[0].cpu().numpy(), lam=m.lam[0].cpu().numpy(),
+               comp=comps[0].cpu().numpy() if want_comp else None)
+    box = ttm.ttm_plan_problem_fft_box(m.plan, 0) if opts.get("path") == ttm.TTM_PATH_FFT else None
+    m.close()
+    return out, box
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("length", [128, 144, 192, 240, 256, 320, 384, 512, 576, 640, 768, 1024])
+def test_long_lines(ttm, length, axis):
+    """One long line along x, y or z, the volume up to three voxels short of it
+    (rows that start on 4, 8 or 16 bytes; columns that end in the padding)."""
+    short = (length // 64 + axis) % 4
+    shape = [18, 21, 23]
+    shape[2 - axis] = length - short
+    wl = synth.make_workload(shape, 7, 3, 2, 1.0, 2, 60, radius=3, seeds=(41, 42, 43))
+    T = o.tensor_template(wl.template, wl.mask, wl.quadrature.astype(np.float64), wl.weights, 2)
+    comp, desc = ttm.build_template(wl.template, wl.mask, 2, wl.quadrature)
+    w_o, C_o = o.ttm_components(wl.volume, T, wl.mask)
+    for precision, tol in ((ttm.TTM_PREC_FP32, TOL), (ttm.TTM_PREC_MIXED, BF16_TOL)):
+        res, box = _maps(ttm, wl.volume, comp, desc, wl.mask, True, path=ttm.TTM_PATH_FFT,
+                         precision=precision)
+        assert box[axis] == length
+        assert np.abs(res["comp"] - C_o).max() <= tol
+        nz = w_o > 0
+        assert np.array_equal(res["w"] > 0, nz)
+        assert (np.abs(res["w"][nz] - w_o[nz]) / w_o[nz]).max() <= 1e-5
+
+
+def _mask(kind, s):
+    m = np.zeros((s, s, s), dtype=np.float32)
+    rng = np.random.default_rng(s)
+    if kind == "ball":
+        m = synth.ball_mask(s)
+    elif kind == "lopsided":             # runs that lie to one side, in few windows
+        m[: s // 2 + 1, s // 2:, : s // 2 + 1] = 1
+        m[0, s - 1, 0] = 0
+    elif kind == "plane":
+        m[s - 1] = 1
+    elif kind == "scattered":            # as many windows as there are runs
+        m = (rng.random((s, s, s)) < 0.4).astype(np.float32)
+    return m
+
+
+@pytest.mark.parametrize("kind", ["ball", "lopsided", "plane", "scattered"])
+@pytest.mark.parametrize("s,shape", [(3, (5, 66, 35)), (6, (40, 9, 33)), (9, (23, 31, 64)),
+                                     (15, (15, 47, 81)), (17, (30, 34, 38))])
+def test_direct_statistics(ttm, s, shape, kind):
+    rng = np.random.default_rng(5)
+    mask = _mask(kind, s)
+    volume = (rng.normal(size=shape) + 3.0).astype(np.float32)
+    q = synth.super_fibonacci_quaternions(8).astype(np.float32)
+    t = rng.normal(size=(s, s, s)).astype(np.float32)
+    comp, desc = ttm.build_template(t, mask, 2, q)
+    res, _ = _maps(ttm, volume, comp, desc, mask, path=ttm.TTM_PATH_DIRECT)
+    w_o = o.local_stats_direct(volume, mask)[2]
+    nz = w_o > 0
+    assert np.array_equal(res["w"] > 0, nz)
+    assert (np.abs(res["w"][nz] - w_o[nz]) / w_o[nz]).max() <= 1e-5
+
+
+@pytest.mark.parametrize("s,n,n_rot,kind,scale", [
+    (3, 2, 700, "ball", 1.0),            # fewer listed voxels than threads
+    (5, 4, 1, "ball", 1.0),              # one node: no room for the tables
+    (8, 4, 37, "ball", 1.0),             # nodes past a multiple of the step
+    (10, 6, 150, "scattered", 1.0),
+    (11, 4, 90, "full", 1.0),            # every voxel: the box build
+    (13, 4, 200, "soft", 1.0),           # weights, not flags
+    (12, 4, 120, "ball", 1e-25),         # squares below the FP32 range
+    (12, 4, 120, "ball", 1e20),          # and above it
+    (12, 8, 64, "lopsided", 1.0),
+    (32, 4, 90, "ball", 1.0),            # two voxels per thread
+    (40, 8, 320, "ball", 1.0),           # four, and few nodes of many voxels
+    (70, 4, 310, "ball", 1.0),           # four at order 4, a ragged last chunk
+])
+def test_template_build(ttm, s, n, n_rot, kind, scale):
+    t = (synth.blob_template(s, 4, seed=s).astype(np.float64) * scale).astype(np.float32)
+    if kind == "soft":
+        mask = synth.soft_ball_mask(s, s // 2, 2.0)
+    else:
+        mask = np.ones((s, s, s), np.float32) if kind == "full" else _mask(kind, s)
+    q = synth.super_fibonacci_quaternions(n_rot).astype(np.float32)
+    comp, desc = ttm.build_template(t, mask, n, q)
+    T = o.tensor_template(t, mask, q.astype(np.float64), np.full(n_rot, 1.0 / n_rot), n)
+    assert desc.mask_sum == pytest.approx(mask.sum(dtype=np.float64))
+    assert np.abs(comp.cpu().numpy() - T).max() <= 2e-5 * np.abs(T).max()
+
+
+@pytest.mark.parametrize("path", ["direct", "fft"])
+@pytest.mark.parametrize("n,shape", [(2, (21, 20, 23)), (4, (23, 19, 37)), (6, (19, 22, 29))])
+def test_candidates_one_by_one(ttm, n, shape, path):
+    """With every candidate refined, one more can only raise lambda, and leaves
+    what the others gave to the bit (whichever one it is refined beside, and
+    however many the search keeps); lambda is phi at q."""
+    wl = synth.make_workload(shape, 9, 3, 1, 1.0, n, 200, radius=4, seeds=(51, 52, 53))
+    T = o.tensor_template(wl.template, wl.mask, wl.quadrature.astype(np.float64), wl.weights, n)
+    comp, desc = ttm.build_template(wl.template, wl.mask, n, wl.quadrature)
+    w_o, C_o = o.ttm_components(wl.volume, T, wl.mask)
+    at = np.argwhere(w_o > 0)[::29]
+    C_pts = C_o[:, at[:, 0], at[:, 1], at[:, 2]].T
+    last = None
+    for k in (1, 2, 3, 4):
+        res, _ = _maps(ttm, wl.volume, comp, desc, wl.mask, n_grid=2048, n_cells=128,
+                       n_candidates=k, n_refined=k,
+                       path={"direct": ttm.TTM_PATH_DIRECT, "fft": ttm.TTM_PATH_FFT}[path])
+        phi = o.phi_unique(C_pts, res["quat"][at[:, 0], at[:, 1], at[:, 2]].astype(np.float64), n)
+        assert np.abs(phi - res["lam"][at[:, 0], at[:, 1], at[:, 2]]).max() <= TOL
+        if last is not None:
+            assert np.all(res["lam"] >= last["lam"])
+            same = res["lam"] == last["lam"]
+            assert np.array_equal(res["quat"][same], last["quat"][same])
+            assert np.array_equal(res["score"], last["score"])
+        last = res
+
+
+@pytest.mark.parametrize("levels", [1, 3, 1000])
+@pytest.mark.parametrize("shape", [(5, 5, 5), (7, 66, 9), (34, 11, 129), (65, 33, 17)])
+def test_peak_lists(ttm, shape, levels):
+    """Scores of one level (a single peak per cube of ties), of few and of
+    many; cubes inside one block of voxels, over many and over the whole map."""
+    Z, Y, X = shape
+    rng = np.random.default_rng(Z)
+    t = synth.blob_template(5, 3, seed=1)
+    mask = synth.ball_mask(5, 2)
+    comp, desc = ttm.build_template(t, mask, 2, synth.super_fibonacci_quaternions(10).astype(np.float32))
+    m = ttm.Matcher([(comp, desc, mask)], [((X, Y, Z), 0)])
+    score = (np.floor(rng.random(shape) * levels) / levels + 0.25).astype(np.float32)
+    quat = np.zeros(shape + (4,), dtype=np.float32)
+    quat[..., 0] = np.arange(score.size, dtype=np.float32).reshape(shape)
+    for radius in (0, 1, 2, 5):
+        for limit in (3, score.size):
+            got = ttm.ttm_extract_peaks(m.plan, 0, _cuda(score), _cuda(quat), _cuda(score), 0.2,
+                                        radius, limit, m.ws)
+            expect = o.extract_peaks(score.astype(np.float64), 0.2, radius, limit)
+            assert np.array_equal((got["z"].astype(np.int64) * Y + got["y"]) * X + got["x"], expect)
+            assert np.array_equal(got["q"][:, 0], quat[..., 0].ravel()[expect])
+            assert np.array_equal(got["lambda"], score.ravel()[expect])
+    m.close()
