@@ -534,56 +534,80 @@ ttm_status launch_spectra_to_bf16(const float2* a, void* b, size_t n, cudaStream
 // (launch_exact_stats).  Large offsets never flag (the mean is removed); a
 // quiet window in a volume of large dynamic range does.
 // Persistent CTAs over x-segments of 128 voxels: the volume statistics and
-// the bounds (FP64 divisions, slow on this GPU) are formed once per CTA; per
-// voxel V and its bound are FP32 (a window that needs more than that is
-// flagged and recomputed in FP64).
-__global__ void __launch_bounds__(128) stats_from_sums_kernel(
+// the bounds are formed once per CTA; per voxel V and its bound are FP32 (a
+// window that needs more than that is flagged and recomputed in FP64).  Small
+// volumes are bound by those FP64 chains, which cost the SM as much for one
+// lane as for 32, hence few CTAs; large ones by instructions (three integer
+// divisions a voxel took as long as its memory), hence coordinates stepped on
+// without division.  STATS_FIGURES
+constexpr int kStatSegs = 2;           // loads of two segments together
+constexpr int kSumThreads = 256, kSumCtas = 6;   // CTAs per SM
+
+__global__ void __launch_bounds__(kSumThreads, kSumCtas) stats_from_sums_kernel(
     const float* __restrict__ s1, const float* __restrict__ s2, float* __restrict__ w, int X,
-    int Y, int Z, int s, double mask_sum, const double* __restrict__ moments, double kappa,
-    unsigned int* __restrict__ flagged) {
-    __shared__ double sh[4];
-    // one warp each for the chains of FP64 divisions and square roots, which
-    // take microseconds here
-    if ((threadIdx.x & 31) == 0) {
+    int Y, int Z, int s, double mask_sum, float fim, const double* __restrict__ moments,
+    double kappa, unsigned int* __restrict__ flagged) {
+    __shared__ double sh[3];
+    // one warp each for the chains of FP64 divisions and square roots
+    if ((threadIdx.x & 31) == 0 && threadIdx.x < 96) {
         const int w = threadIdx.x >> 5;
         const double nv = (double)X * Y * Z;
         const double eps = 5.9604644775390625e-8;          // 2^-24
-        if (w == 0) sh[0] = 1.0 / mask_sum;
-        if (w == 1 || w == 2) {
+        if (w < 2) {
             const double mean = moments[0] / nv;
             const double var_f = fmax(moments[1] / nv - mean * mean, 0.0);
-            if (w == 1) sh[1] = 1e-6 * mask_sum * var_f;
-            else sh[2] = kappa * eps * mask_sum * sqrt(var_f);       // bound on |dS1|
+            if (w == 0) sh[0] = 1e-6 * mask_sum * var_f;
+            else sh[1] = kappa * eps * mask_sum * sqrt(var_f);       // bound on |dS1|
         }
-        if (w == 3) sh[3] = kappa * eps * mask_sum * sqrt(fmax(moments[2], 0.0) / nv);   // on |dS2|
+        if (w == 2) sh[2] = kappa * eps * mask_sum * sqrt(fmax(moments[2], 0.0) / nv);   // on |dS2|
     }
     __syncthreads();
-    const float fim = (float)sh[0], ffl = (float)sh[1], fe1 = (float)sh[2], fe2 = (float)sh[3];
+    const float ffl = (float)sh[0], fe1 = (float)sh[1], fe2 = (float)sh[2];
+    // segment first, first + step, ...: neighbours in a CTA are neighbours in
+    // memory; (xs, y, z) and the step as digits in base (xt, Y)
     const uint32_t xt = (uint32_t)((X + 127) / 128);
-    const uint32_t segs = xt * (uint32_t)Y * (uint32_t)Z;
+    const uint32_t step = gridDim.x * (kSumThreads / 128);
+    const uint32_t first = blockIdx.x * (kSumThreads / 128) + threadIdx.x / 128;
+    const uint32_t frow = first / xt, srow = step / xt;
+    int xs = (int)(first - frow * xt), y = (int)(frow % (uint32_t)Y), z = (int)(frow / (uint32_t)Y);
+    const int dx = (int)(step - srow * xt), dy = (int)(srow % (uint32_t)Y), dz = (int)(srow / (uint32_t)Y);
     unsigned int nflag = 0;
-    for (uint32_t sg = blockIdx.x; sg < segs; sg += gridDim.x) {
-        const uint32_t row = sg / xt;
-        const int x = (int)(sg - row * xt) * 128 + threadIdx.x;
-        const int y = (int)(row % (uint32_t)Y), z = (int)(row / (uint32_t)Y);
-        if (x >= X) continue;
-        const size_t v = ((size_t)z * Y + y) * X + x;
-        float out = 0.f;
-        if (interior(x, X, s) && interior(y, Y, s) && interior(z, Z, s)) {
-            // V in FP32; its own rounding (eps (S2 + S1^2/m)) joins the bound
-            const float S1 = s1[v], S2 = s2[v];
-            const float q = S1 * S1 * fim;
-            const float V = S2 - q;
-            const float dv = fe2 + (2.f * fabsf(S1) * fe1 + fe1 * fe1) * fim +
-                             1.2e-7f * (fabsf(S2) + q);
-            if (dv > 2e-5f * V || fabsf(V - ffl) <= dv) {
-                out = -1.f;
-                ++nflag;
-            } else if (V > ffl) {
-                out = rsqrtf(V);
-            }
+    while (z < Z) {
+        size_t v[kStatSegs];
+        float S1[kStatSegs], S2[kStatSegs];
+        bool on[kStatSegs], in[kStatSegs];
+#pragma unroll
+        for (int k = 0; k < kStatSegs; ++k) {
+            const int x = xs * 128 + (threadIdx.x & 127);
+            on[k] = z < Z && x < X;
+            in[k] = on[k] && interior(x, X, s) && interior(y, Y, s) && interior(z, Z, s);
+            v[k] = ((size_t)z * Y + y) * X + x;
+            S1[k] = in[k] ? __ldg(s1 + v[k]) : 0.f;
+            S2[k] = in[k] ? __ldg(s2 + v[k]) : 0.f;
+            xs += dx;
+            y += dy;
+            z += dz;
+            if (xs >= (int)xt) { xs -= (int)xt; ++y; }
+            if (y >= Y) { y -= Y; ++z; }
         }
-        w[v] = out;
+#pragma unroll
+        for (int k = 0; k < kStatSegs; ++k) {
+            float out = 0.f;
+            if (in[k]) {
+                // V in FP32; its own rounding (eps (S2 + S1^2/m)) joins the bound
+                const float q = S1[k] * S1[k] * fim;
+                const float V = S2[k] - q;
+                const float dv = fe2 + (2.f * fabsf(S1[k]) * fe1 + fe1 * fe1) * fim +
+                                 1.2e-7f * (fabsf(S2[k]) + q);
+                if (dv > 2e-5f * V || fabsf(V - ffl) <= dv) {
+                    out = -1.f;
+                    ++nflag;
+                } else if (V > ffl) {
+                    out = rsqrtf(V);
+                }
+            }
+            if (on[k]) w[v[k]] = out;
+        }
     }
     for (int o = 16; o > 0; o >>= 1) nflag += __shfl_down_sync(0xffffffffu, nflag, o);
     if ((threadIdx.x & 31) == 0 && nflag) atomicAdd(flagged, nflag);
@@ -594,10 +618,11 @@ ttm_status launch_stats_from_sums(const float* s1, const float* s2, float* w, in
                                   unsigned int* flagged, cudaStream_t st, long long* cnt) {
     const size_t segs = (size_t)((X + 127) / 128) * Y * Z;
     if (segs > 0xFFFFFFFFull) return TTM_ERR_UNSUPPORTED;
-    const unsigned grid = (unsigned)(segs < 152 * 16 ? segs : 152 * 16);
+    const size_t per = kStatSegs * (kSumThreads / 128), ctas = (segs + per - 1) / per;
+    const unsigned grid = (unsigned)(ctas < 152 * kSumCtas ? ctas : 152 * kSumCtas);
     const double kappa = 2.0 * std::log2((double)X * Y * Z);
-    stats_from_sums_kernel<<<grid, 128, 0, st>>>(s1, s2, w, X, Y, Z, s, mask_sum, moments, kappa,
-                                                 flagged);
+    stats_from_sums_kernel<<<grid, kSumThreads, 0, st>>>(
+        s1, s2, w, X, Y, Z, s, mask_sum, (float)(1.0 / mask_sum), moments, kappa, flagged);
     return after_launch(cnt);
 }
 
@@ -611,7 +636,7 @@ static bool box_cols_ok(int L, int B) {
 // part of its padded volume, so only the s^2 rows that meet it are transformed
 // along x, only its s planes along y, and the z pass reads only those planes;
 // the zeros around it are neither written nor read, and all K boxes go through
-// three launches (a 24^3 box in 192 x 160 x 128: 66 -> 9 us per box).
+// three launches (a 24^3 box in 192 x 160 x 128: 65 -> 6 us per box).
 ttm_status launch_template_spectra(const float* comp, int K, int s, const FftShape& S,
                                    float* pad, float2* tspec, cudaStream_t st, long long* cnt) {
     FftGeom g{S.Xp, S.Yp, S.Zp, spec_pitch(S.Xp)};
