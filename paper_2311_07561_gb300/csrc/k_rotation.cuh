@@ -384,10 +384,9 @@ __device__ __forceinline__ F2 f2_dot(const F2 (&a)[4], const F2 (&b)[4]) {
     return f2_fma(a[3], b[3], f2_fma(a[2], b[2], f2_fma(a[0], b[0], f2_mul(a[1], b[1]))));
 }
 
-// grad_at for two points
+// the gradient of grad_at for two points (its lam is f2_dot(x, g))
 template <int N>
-__device__ __forceinline__ void grad2_at(const F2 (&C)[Geo<N>::K], const F2 (&x)[4], F2 (&g)[4],
-                                         F2& lam) {
+__device__ __forceinline__ void grad2_at(const F2 (&C)[Geo<N>::K], const F2 (&x)[4], F2 (&g)[4]) {
     constexpr GradTab<N> T{};
     Monomials2<N - 1> mg;
     monomials2<N - 1>(x, mg);
@@ -400,7 +399,6 @@ __device__ __forceinline__ void grad2_at(const F2 (&C)[Geo<N>::K], const F2 (&x)
 #pragma unroll
         for (int i = 0; i < 4; ++i) g[i] = f2_fma(mw, C[T.comp[i][b]], g[i]);
     }
-    lam = f2_dot(x, g);
 }
 
 // eval_at for two points; h = the 10 entries of H
@@ -441,11 +439,15 @@ __device__ __forceinline__ void power_steps2(const F2 (&C)[Geo<N>::K], float sig
                                              F2& lam, bool want_lam) {
     const F2 sig = f2(sigma, sigma);
     F2 g[4];
+    lam = f2(0.f, 0.f);
 #pragma unroll 1
     for (int s = 0; s < 3; ++s) {
         if (s == 2 && !want_lam) break;
-        grad2_at<N>(C, x, g, lam);
-        if (s == 2) break;
+        grad2_at<N>(C, x, g);
+        if (s == 2) {
+            lam = f2_dot(x, g);
+            break;
+        }
 #pragma unroll
         for (int i = 0; i < 4; ++i) x[i] = f2_fma(sig, x[i], g[i]);
         normalise2(x);
@@ -547,8 +549,10 @@ __device__ __forceinline__ void refine2(const F2 (&C)[Geo<N>::K], float sigma, i
         const bool last = it + 1 == iters;
         F2 h[10], g[4], lam;
         // the last trial needs only phi (see refine)
-        if (N >= 6 && last && it > 0) grad2_at<N>(C, xt, g, lam);
-        else eval2_at<N>(C, xt, h, g, lam);
+        if (N >= 6 && last && it > 0) {
+            grad2_at<N>(C, xt, g);
+            lam = f2_dot(xt, g);
+        } else eval2_at<N>(C, xt, h, g, lam);
         const float va = f2_get(lam, 0), vb = f2_get(lam, 1);
         const bool keep_a = !(ta && va < la - eps), keep_b = !(tb && vb < lb - eps);
 #pragma unroll
