@@ -307,6 +307,16 @@ bool fixed_cols_mul(int L, const float2* spec, const float2* tspec, float2* prod
     }
 }
 
+bool fixed_cols_mul_box(int L, const float2* spec, const float2* box, float2* prod, int Bz, int K,
+                        const float2* tw, int lo, int hi, ColsIn ci, cudaStream_t st, cudaError_t* err) {
+    switch (L) {
+#define C(L) TTM_FFT_CASE(L, cols_mul_box(spec, box, prod, Bz, K, tw, lo, hi, ci, st))
+        TTM_FFT_LENGTHS(C)
+#undef C
+        default: return false;
+    }
+}
+
 bool fixed_cols_mul(int L, const float2* spec, const __nv_bfloat162* tspec, __nv_bfloat162* prod,
                     int Bz, int K, const float2* tw, int lo, int hi, cudaStream_t st,
                     cudaError_t* err) {
@@ -632,6 +642,36 @@ static bool box_cols_ok(int L, int B) {
     return fft_template_length(L) && (B % 8 == 0 || L < 144 || L == 256);
 }
 
+static bool box_rows_ok(const FftShape& S) {
+    const int Xh = spec_pitch(S.Xp);
+    return fft_template_length(S.Xp) && box_cols_ok(S.Yp, Xh) && box_cols_ok(S.Zp, S.Yp * Xh);
+}
+
+// lengths and batches of the packed multiply over boxes
+static bool fft_box_mul_ok(int L, int Bz, int K) {
+    switch (L) {
+#define C(L) case L: return fftk::mulp_takes<L, float2>(Bz, K);
+        TTM_FFT_LENGTHS(C)
+#undef C
+        default: return false;
+    }
+}
+
+// K boxes through the x and y passes: their s planes in tspec
+static ttm_status box_planes(const float* comp, int K, int s, const FftShape& S, float2* tspec,
+                             cudaStream_t st, long long* cnt) {
+    FftGeom g{S.Xp, S.Yp, S.Zp, spec_pitch(S.Xp)};
+    const int c = s / 2;
+    cudaError_t err = cudaSuccess;
+    fixed_rows_r2c(S.Xp, comp, s, s, s, g, tspec, S.d_tw_x, 0, nullptr, BoxIn{s, c, K}, st, &err);
+    TTM_CUDA_TRY(err);
+    TTM_TRY(after_launch(cnt));
+    const ColsMap my{0, s, S.Zp, S.Zp - c, 0, S.Yp - 1};
+    fixed_cols(S.Yp, tspec, g.Xh, K * s, my, S.d_tw_y, -1, st, &err, ColsIn{c, s, 1.f});
+    TTM_CUDA_TRY(err);
+    return after_launch(cnt);
+}
+
 // K boxes of edge s -> their half spectra, scaled by 1/N.  A box is a small
 // part of its padded volume, so only the s^2 rows that meet it are transformed
 // along x, only its s planes along y, and the z pass reads only those planes;
@@ -644,15 +684,10 @@ ttm_status launch_template_spectra(const float* comp, int K, int s, const FftSha
     const size_t nspec = S.nspec();
     const int s3 = s * s * s, c = s / 2;
     const float scale = 1.0f / (float)nreal;
-    if (fft_template_length(S.Xp) && box_cols_ok(S.Yp, g.Xh) && box_cols_ok(S.Zp, S.Yp * g.Xh)) {
+    if (box_rows_ok(S)) {
+        TTM_TRY(box_planes(comp, K, s, S, tspec, st, cnt));
         cudaError_t err = cudaSuccess;
-        fixed_rows_r2c(S.Xp, comp, s, s, s, g, tspec, S.d_tw_x, 0, nullptr, BoxIn{s, c, K}, st, &err);
-        TTM_CUDA_TRY(err);
-        TTM_TRY(after_launch(cnt));
-        const ColsMap my{0, s, S.Zp, S.Zp - c, 0, S.Yp - 1}, mz{0, 1, 1, 0, 0, S.Zp - 1};
-        fixed_cols(S.Yp, tspec, g.Xh, K * s, my, S.d_tw_y, -1, st, &err, ColsIn{c, s, 1.f});
-        TTM_CUDA_TRY(err);
-        TTM_TRY(after_launch(cnt));
+        const ColsMap mz{0, 1, 1, 0, 0, S.Zp - 1};
         fixed_cols(S.Zp, tspec, S.Yp * g.Xh, K, mz, S.d_tw_z, -1, st, &err, ColsIn{c, s, scale});
         TTM_CUDA_TRY(err);
         return after_launch(cnt);
@@ -668,6 +703,26 @@ ttm_status launch_template_spectra(const float* comp, int K, int s, const FftSha
         TTM_TRY(after_launch(cnt));
     }
     return TTM_OK;
+}
+
+// launch_template_spectra and launch_fft_spectrum_inverse_z of K boxes used
+// once: the boxes' z pass, the multiply and the inverse z pass are one launch
+// where the packed multiply applies, the template spectra stay on the chip.
+ttm_status launch_box_spectrum_inverse_z(const float* comp, int K, int s, const FftShape& S, float* pad,
+                                         const float2* spec, float2* tspec, float2* prod,
+                                         const FftKeep& keep, cudaStream_t st, long long* cnt) {
+    const int Bz = S.Yp * spec_pitch(S.Xp);
+    if (box_rows_ok(S) && fft_box_mul_ok(S.Zp, Bz, K)) {
+        TTM_TRY(box_planes(comp, K, s, S, tspec, st, cnt));
+        cudaError_t err = cudaSuccess;
+        const float scale = 1.0f / (float)((size_t)S.Xp * S.Yp * S.Zp);
+        fixed_cols_mul_box(S.Zp, spec, tspec, prod, Bz, K, S.d_tw_z, keep.z0, keep.z1,
+                           ColsIn{s / 2, s, scale}, st, &err);
+        TTM_CUDA_TRY(err);
+        return after_launch(cnt);
+    }
+    TTM_TRY(launch_template_spectra(comp, K, s, S, pad, tspec, st, cnt));
+    return launch_fft_spectrum_inverse_z(spec, tspec, K, S, prod, keep, st, cnt);
 }
 
 }  // namespace ttm

@@ -736,6 +736,8 @@ struct FftLen {
                                int sign, cudaStream_t st);
     static cudaError_t cols_mul(const float2* spec, const float2* tspec, float2* prod, int Bz, int K,
                                 const float2* tw, int lo, int hi, cudaStream_t st);
+    static cudaError_t cols_mul_box(const float2* spec, const float2* box, float2* prod, int Bz, int K,
+                                    const float2* tw, int lo, int hi, ColsIn ci, cudaStream_t st);
     static cudaError_t cols_mul_bf(const float2* spec, const __nv_bfloat162* tspec,
                                    __nv_bfloat162* prod, int Bz, int K, const float2* tw, int lo,
                                    int hi, cudaStream_t st);
@@ -833,29 +835,39 @@ cudaError_t run_cols(PS* d, int B, int na, ColsMap mp, const float2* tw, cudaStr
     }
 }
 
+// the packed multiply of K components (BOX: of their boxes before the z pass)
+template <int L, typename TS, typename PS, bool BOX>
+cudaError_t run_mulp(const float2* spec, const TS* tspec, PS* prod, int Bz, int K, const float2* tw,
+                     int lo, int hi, ColsIn ci, cudaStream_t st) {
+    using Plan = MulPlan<L, TS>;
+    constexpr int L1 = PackSplit<L>::L1, L2 = PackSplit<L>::L2, NP = Plan::NP, MS = Plan::MS;
+    constexpr size_t smem = mulp_smem<L1, L2, NP, MS, TS, BOX>();
+    constexpr int threads = L1 * NP * mulp_teams<L1, L2, NP, MS, TS, BOX>();
+    static_assert(threads > 0, "at least one team");
+    auto kern = mulp_t<L1, L2, NP, MS, TS, PS, BOX>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int sms = 0;
+    if ((e = sm_count(&sms)) != cudaSuccess) return e;
+    const unsigned ntiles = (unsigned)(Bz / (2 * NP));
+    const unsigned grid = ntiles < (unsigned)sms ? ntiles : (unsigned)sms;
+    kern<<<grid, threads, smem, st>>>(spec, tspec, prod, Bz, K, tw, lo, hi, ntiles, ci);
+    return cudaGetLastError();
+}
+
+// one or two lines per column (the window sums): a CTA's teams would idle (144,
+// one component: scalar 37 us, packed 44)
+template <int L, typename TS> bool mulp_takes(int Bz, int K) {
+    if constexpr (mul_packed<L, TS>()) return K > 2 && Bz % (2 * MulPlan<L, TS>::NP) == 0;
+    return false;
+}
+
 template <int L, typename TS, typename PS>
 cudaError_t run_cols_mul(const float2* spec, const TS* tspec, PS* prod, int Bz, int K,
                          const float2* tw, int lo, int hi, cudaStream_t st) {
     if constexpr (mul_packed<L, TS>()) {
-        // one or two lines per column (the window sums): a CTA's teams would
-        // idle (144, one component: scalar 37 us, packed 44)
-        using Plan = MulPlan<L, TS>;
-        if (K > 2 && Bz % (2 * Plan::NP) == 0) {
-            constexpr int L1 = PackSplit<L>::L1, L2 = PackSplit<L>::L2, NP = Plan::NP, MS = Plan::MS;
-            constexpr size_t smem = mulp_smem<L1, L2, NP, MS, TS>();
-            constexpr int threads = L1 * NP * mulp_teams<L1, L2, NP, MS, TS>();
-            static_assert(threads > 0, "at least one team");
-            auto kern = mulp_t<L1, L2, NP, MS, TS, PS>;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
-            if (e != cudaSuccess) return e;
-            int sms = 0;
-            if ((e = sm_count(&sms)) != cudaSuccess) return e;
-            const unsigned ntiles = (unsigned)(Bz / (2 * NP));
-            const unsigned grid = ntiles < (unsigned)sms ? ntiles : (unsigned)sms;
-            kern<<<grid, threads, smem, st>>>(spec, tspec, prod, Bz, K, tw, lo, hi, ntiles);
-            return cudaGetLastError();
-        }
+        if (mulp_takes<L, TS>(Bz, K))
+            return run_mulp<L, TS, PS, false>(spec, tspec, prod, Bz, K, tw, lo, hi, ColsIn{0, L, 1.f}, st);
     }
     if constexpr (two_level<L>()) {
         constexpr int L1 = MulSplit<L>::L1, L2 = MulSplit<L>::L2;
@@ -1030,6 +1042,17 @@ template <int L>
 cudaError_t FftLen<L>::cols_mul(const float2* spec, const float2* tspec, float2* prod, int Bz,
                                 int K, const float2* tw, int lo, int hi, cudaStream_t st) {
     return fftk::run_cols_mul<L, float2, float2>(spec, tspec, prod, Bz, K, tw, lo, hi, st);
+}
+
+// cudaErrorNotSupported where the packed multiply does not apply
+template <int L>
+cudaError_t FftLen<L>::cols_mul_box(const float2* spec, const float2* box, float2* prod, int Bz, int K,
+                                    const float2* tw, int lo, int hi, ColsIn ci, cudaStream_t st) {
+    if constexpr (fftk::mul_packed<L, float2>()) {
+        if (fftk::mulp_takes<L, float2>(Bz, K))
+            return fftk::run_mulp<L, float2, float2, true>(spec, box, prod, Bz, K, tw, lo, hi, ci, st);
+    }
+    return cudaErrorNotSupported;
 }
 
 template <int L>

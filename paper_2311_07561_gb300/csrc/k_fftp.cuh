@@ -392,40 +392,48 @@ template <int L, typename TS> struct MulPlan {
                                  : (L == 128 || L == 288 || L == 320 || L == 480 ? 1 : 2);
     static constexpr bool on = bf ? L <= 512 : L <= 480;
 };
+// BOX: the template lines come as they are before their own z transform (a
+// rotated template's box: len planes, the rest zero).  The team transforms a
+// line forward, multiplies, and goes on, the products where the samples were:
+// the template spectra are neither written nor read (128 points, boxes of 24,
+// 501 lines a column: 2152 us of z pass and 2622 of multiply -> 3276).
 // Persistent CTAs over column tiles; the teams of a CTA (L1 NP threads with
 // a named barrier each) share the tile's image samples in shared memory (the
 // next tile's arrive meanwhile) and take the components in turn.
 template <int L1, int L2, int NP, int MS, typename TS> constexpr size_t mulp_team() {
     return (size_t)L1 * L2 * 2 * NP * sizeof(TS) * MS + c2_exchange<L1, L2, NP>();
 }
-template <int L1, int L2, int NP> constexpr size_t mulp_shared() {
-    return (size_t)L1 * L2 * (2 * 2 * NP * sizeof(float2) + 16);     // two image tiles, twiddles
+template <int L1, int L2, int NP, bool BOX> constexpr size_t mulp_shared() {
+    // two image tiles, twiddles
+    return (size_t)L1 * L2 * (2 * 2 * NP * sizeof(float2) + (BOX ? 32 : 16));
 }
-template <int L1, int L2, int NP, int MS, typename TS> constexpr int mulp_teams() {
+template <int L1, int L2, int NP, int MS, typename TS, bool BOX = false> constexpr int mulp_teams() {
     constexpr size_t room = (size_t)226 * 1024;
-    constexpr int by_smem = mulp_shared<L1, L2, NP>() < room
-        ? (int)((room - mulp_shared<L1, L2, NP>()) / mulp_team<L1, L2, NP, MS, TS>()) : 0;
+    constexpr int by_smem = mulp_shared<L1, L2, NP, BOX>() < room
+        ? (int)((room - mulp_shared<L1, L2, NP, BOX>()) / mulp_team<L1, L2, NP, MS, TS>()) : 0;
     constexpr int by_regs = 65536 / (L1 * NP * ((c2_regs<L1, L2>() + 7) / 8 * 8));
     constexpr int n = by_smem < by_regs ? by_smem : by_regs;
     return n > 8 ? 8 : n;
 }
-template <int L1, int L2, int NP, int MS, typename TS> constexpr size_t mulp_smem() {
-    return mulp_shared<L1, L2, NP>() + mulp_teams<L1, L2, NP, MS, TS>() * mulp_team<L1, L2, NP, MS, TS>();
+template <int L1, int L2, int NP, int MS, typename TS, bool BOX = false> constexpr size_t mulp_smem() {
+    return mulp_shared<L1, L2, NP, BOX>() +
+           mulp_teams<L1, L2, NP, MS, TS, BOX>() * mulp_team<L1, L2, NP, MS, TS>();
 }
 
-template <int L1, int L2, int NP, int MS, typename TS, typename PS>
-__global__ void __launch_bounds__(L1 * NP * mulp_teams<L1, L2, NP, MS, TS>(), 1) mulp_t(
+template <int L1, int L2, int NP, int MS, typename TS, typename PS, bool BOX>
+__global__ void __launch_bounds__(L1 * NP * mulp_teams<L1, L2, NP, MS, TS, BOX>(), 1) mulp_t(
     const float2* __restrict__ spec, const TS* __restrict__ tspec, PS* __restrict__ out, int B, int K,
-    const float2* __restrict__ tw, int lo, int hi, uint32_t ntiles) {
+    const float2* __restrict__ tw, int lo, int hi, uint32_t ntiles, ColsIn ci) {
     constexpr int L = L1 * L2;
     constexpr int T = L1 * NP, TB = 2 * NP;
-    constexpr int kTeams = mulp_teams<L1, L2, NP, MS, TS>();
+    constexpr int kTeams = mulp_teams<L1, L2, NP, MS, TS, BOX>();
     constexpr int kSegF = TB * (int)sizeof(float2) / 16, kSegT = TB * (int)sizeof(TS) / 16;
     extern __shared__ __align__(16) unsigned char smp[];
     float4* tws = reinterpret_cast<float4*>(smp);
-    float2* img = reinterpret_cast<float2*>(smp + (size_t)L * 16);          // two tiles
+    const float4* twf = tws + L;                                            // BOX: forward
+    float2* img = reinterpret_cast<float2*>(smp + (size_t)L * (BOX ? 32 : 16));   // two tiles
     const int team = threadIdx.x / T, t = threadIdx.x % T;
-    unsigned char* mine = smp + mulp_shared<L1, L2, NP>() + team * mulp_team<L1, L2, NP, MS, TS>();
+    unsigned char* mine = smp + mulp_shared<L1, L2, NP, BOX>() + team * mulp_team<L1, L2, NP, MS, TS>();
     float4* zx = reinterpret_cast<float4*>(mine);
     TS* st = reinterpret_cast<TS*>(mine + c2_exchange<L1, L2, NP>());
     const int n1 = t / NP, pair = t % NP;
@@ -444,9 +452,11 @@ __global__ void __launch_bounds__(L1 * NP * mulp_teams<L1, L2, NP, MS, TS>(), 1)
     auto copy_comp = [&](uint32_t tile, int k, int buf) {
         const TS* src = tspec + (size_t)k * plane + (size_t)tile * TB;
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(st + (size_t)buf * L * TB);
-        for (int e = t; e < L * kSegT; e += T) {
-            const int l = e / kSegT, seg = e % kSegT;
-            cp_async16(dst + (uint32_t)(e * 16), reinterpret_cast<const char*>(src + (size_t)l * B) + seg * 16);
+        for (int e = t; e < (BOX ? ci.len : L) * kSegT; e += T) {
+            const int seg = e % kSegT;
+            int l = e / kSegT - (BOX ? ci.c : 0);
+            if (l < 0) l += L;
+            cp_async16(dst + (uint32_t)((l * kSegT + seg) * 16), reinterpret_cast<const char*>(src + (size_t)l * B) + seg * 16);
         }
     };
     uint32_t tile = blockIdx.x;
@@ -469,6 +479,7 @@ __global__ void __launch_bounds__(L1 * NP * mulp_teams<L1, L2, NP, MS, TS>(), 1)
 #pragma unroll
     for (int q = 0; q < MS; ++q) copy_next();
     fill_tw<+1>(tws, tw, L, threadIdx.x, T * kTeams);
+    if constexpr (BOX) fill_tw<-1>(tws + L, tw, L, threadIdx.x, T * kTeams);
     int buf = 0, cur = 0;
     for (; tile < ntiles; tile += gridDim.x, buf ^= 1) {
         const bool more = tile + gridDim.x < ntiles;
@@ -480,17 +491,46 @@ __global__ void __launch_bounds__(L1 * NP * mulp_teams<L1, L2, NP, MS, TS>(), 1)
         for (int k = team; k < K; k += kTeams) {
             asm volatile("cp.async.wait_group %0;\n" ::"n"(MS - 1) : "memory");
             sync_team();                 // the component in place, the exchange free
+            TS* in = st + (size_t)cur * L * TB;
+            auto product = [&](int at, C2 q) {            // F(f) conj(q) of two columns
+                const float4 f = *reinterpret_cast<const float4*>(im + at);
+                const float2 a = cmulc(make_float2(f.x, f.y), make_float2(f2_get(q.re, 0), f2_get(q.im, 0)));
+                const float2 b = cmulc(make_float2(f.z, f.w), make_float2(f2_get(q.re, 1), f2_get(q.im, 1)));
+                return C2{f2(a.x, b.x), f2(a.y, b.y)};
+            };
+            if constexpr (BOX) {
+                {
+                    C2 v[L2];
+#pragma unroll
+                    for (int n2 = 0; n2 < L2; ++n2) {
+                        const int l = n1 + L1 * n2, d = l + ci.c >= L ? l + ci.c - L : l + ci.c;
+                        v[n2] = d < ci.len ? c2_load(in + l * TB + 2 * pair) : C2{dup2(0.f), dup2(0.f)};
+                    }
+                    c2_step_a<L1, L2, -1, NP>(v, zx, twf, n1, pair);
+                }
+                sync_team();
+                const F2 sc = dup2(ci.scale);
+#pragma unroll 1
+                for (int it = t; it < L2 * NP; it += T) {
+                    const int k2 = it / NP, pb = it % NP;
+                    C2 u[L1];
+                    c2_step_b<L1, -1, NP>(u, zx, k2, pb);
+#pragma unroll
+                    for (int k1 = 0; k1 < L1; ++k1) {
+                        const int at = (k2 + L2 * k1) * TB + 2 * pb;
+                        if (ci.scale != 1.f) u[k1] = C2{f2_mul(u[k1].re, sc), f2_mul(u[k1].im, sc)};
+                        c2_store(in + at, product(at, u[k1]));
+                    }
+                }
+                sync_team();             // the products in place, the exchange free
+            }
             {
-                const TS* in = st + (size_t)cur * L * TB;
                 C2 v[L2];
 #pragma unroll
                 for (int n2 = 0; n2 < L2; ++n2) {
                     const int at = (n1 + L1 * n2) * TB + 2 * pair;
-                    const float4 f = *reinterpret_cast<const float4*>(im + at);
-                    const C2 q = c2_load(in + at);
-                    const float2 a = cmulc(make_float2(f.x, f.y), make_float2(f2_get(q.re, 0), f2_get(q.im, 0)));
-                    const float2 b = cmulc(make_float2(f.z, f.w), make_float2(f2_get(q.re, 1), f2_get(q.im, 1)));
-                    v[n2] = C2{f2(a.x, b.x), f2(a.y, b.y)};
+                    if constexpr (BOX) v[n2] = c2_load(in + at);
+                    else v[n2] = product(at, c2_load(in + at));
                 }
                 c2_step_a<L1, L2, +1, NP>(v, zx, tws, n1, pair);
             }

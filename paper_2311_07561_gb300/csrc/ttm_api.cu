@@ -1591,13 +1591,11 @@ ttm_status ttm_classical_ncc(ttm_plan_t plan, int problem, const float* d_templa
     for (int j0 = 0; j0 < n_rot; j0 += kClassicalBatch) {
         const int nb = std::min(kClassicalBatch, n_rot - j0);
         TTM_TRY(timed(plan, KC_TEMPLATE, st, [&] {
-            TTM_TRY(launch_rotate_normalise(d_template, T.d_mask, s, d_quats, j0, nb, rot,
-                                            T.desc.mask_sum, d_bad, st, &plan->launches));
-            return launch_template_spectra(rot, nb, s, pr.fft, pad, tspec, st, &plan->launches);
+            return launch_rotate_normalise(d_template, T.d_mask, s, d_quats, j0, nb, rot,
+                                           T.desc.mask_sum, d_bad, st, &plan->launches);
         }));
         TTM_TRY(timed(plan, KC_FFT_SPECTRUM, st, [&] {
-            return launch_fft_spectrum_inverse_z(spec, tspec, nb, pr.fft, prod,
-                                                 keep, st,
+            return launch_box_spectrum_inverse_z(rot, nb, s, pr.fft, pad, spec, tspec, prod, keep, st,
                                                  &plan->launches);
         }));
         TTM_TRY(timed(plan, KC_FFT_INVERSE, st, [&] {

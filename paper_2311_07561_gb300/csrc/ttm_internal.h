@@ -375,6 +375,9 @@ ttm_status launch_fft_spectrum_inverse_z(const float2* spec, const float2* tspec
 ttm_status launch_fft_inverse_yx(float2* prod, int K, int X, int Y, int Z, const FftShape& S,
                                  float* corr, int* status, const FftKeep& keep, cudaStream_t st,
                                  long long* cnt);
+ttm_status launch_box_spectrum_inverse_z(const float* comp, int K, int s, const FftShape& S, float* pad,
+                                         const float2* spec, float2* tspec, float2* prod,
+                                         const FftKeep& keep, cudaStream_t st, long long* cnt);
 ttm_status launch_template_spectra(const float* comp, int K, int s, const FftShape& S,
                                    float* pad, float2* tspec, cudaStream_t st, long long* cnt);
 

@@ -187,3 +187,35 @@ def test_peak_lists(ttm, shape, levels):
             assert np.array_equal(got["q"][:, 0], quat[..., 0].ravel()[expect])
             assert np.array_equal(got["lambda"], score.ravel()[expect])
     m.close()
+
+
+@pytest.mark.parametrize("depth,s,n_rot", [(125, 9, 3), (141, 8, 34), (192, 15, 5), (239, 12, 2), (460, 9, 4)])
+def test_classical_long_z(ttm, depth, s, n_rot):
+    """Classical matching where a rotated template's own z transform runs
+    inside the multiply (long z lines, three rotations and more in a batch; 34
+    leaves a batch of two, which takes the passes one by one)."""
+    import torch
+    rng = np.random.default_rng(depth)
+    shape = (depth, 23, 26)
+    volume = rng.normal(size=shape).astype(np.float32)
+    t, mask = synth.blob_template(s, 4, seed=s), synth.ball_mask(s)
+    q = synth.shoemake_quaternions(n_rot, 4).astype(np.float32)
+    comp, desc = ttm.build_template(t, mask, 2, synth.super_fibonacci_quaternions(20).astype(np.float32))
+    po = ttm.PlanOpts()
+    po.path = ttm.TTM_PATH_FFT
+    m = ttm.Matcher([(comp, desc, mask)], [(shape[::-1], 0)], opts=po)
+    vol = _cuda(volume)
+    m.run([vol])
+    best = torch.empty(shape, dtype=torch.float32, device="cuda")
+    arg = torch.empty(shape, dtype=torch.int32, device="cuda")
+    ws = torch.empty(ttm.ttm_classical_workspace_size(m.plan, 0), dtype=torch.uint8, device="cuda")
+    ttm.ttm_classical_ncc(m.plan, 0, _cuda(t), _cuda(q), n_rot, vol, m.w[0], best, arg, ws)
+    torch.cuda.synchronize()
+    best, arg = best.cpu().numpy(), arg.cpu().numpy()
+    m.close()
+    c = o.classical_ncc(volume, t, mask, q.astype(np.float64))
+    keep = o.interior_mask(shape, s)
+    best_o = np.where(keep, c.max(axis=0), 0.0)
+    assert np.abs(best - best_o).max() <= TOL
+    zi, yi, xi = np.nonzero(keep)
+    assert np.all(c[arg[zi, yi, xi], zi, yi, xi] >= best_o[zi, yi, xi] - TOL)
