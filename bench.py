@@ -592,7 +592,7 @@ def stage_traffic(name: str, K: int, storage: str, n_int: int):
 
 
 # the score + rotation step runs as two kernel classes (grid search and
-# refinement) on two streams; its roofline is taken over both
+# refinement); its roofline is taken over both
 STAGE_CLASSES = {"score_rotation": ("rotation_search", "rotation_polish")}
 
 
@@ -609,9 +609,8 @@ def roofline(kernels: dict, steps: int, geo: dict, peaks: dict) -> dict:
     count), bytes for the memory-bound stages (what each pass must read and
     write at the plan's storage precision), never a count of what the kernel
     happens to execute.  The score + rotation stage is timed by its span
-    (rotation_stage: the wall time of the stage on the launch stream, its
-    search and refinement overlapping on two streams), else as the sum of its
-    two kernel classes' CUDA-event times (an upper bound)."""
+    (rotation_stage: the wall time of the stage on the launch stream), else as
+    the sum of its two kernel classes' CUDA-event times (an upper bound)."""
     K, nvox, n_int = geo["K"], geo["nvox"], geo["n_interior"]
     per_step = {k: v["ms"] / steps for k, v in kernels.items()}
     span = per_step.pop("rotation_stage", None)

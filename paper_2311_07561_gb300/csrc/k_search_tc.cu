@@ -33,7 +33,9 @@
 // What bounds it: the integer ALU of the reduction, 1.5 operations per value
 // (one LOP3 to pack the key, half a three-input maximum), 64 lanes a clock:
 // 3.5 clocks per 128-lane column measured alone, 4.1 with two regions kept
-// and 5.0 with eight; the MMAs take 1.5 (KP = 48) or 3 (KP = 96).  With every
+// and 5.0 with eight (sixteen reducing warps of 80 registers, which is all that
+// six warps on a scheduler leave each, were no faster: 512 x 512 x 256 in 28.6
+// ms against 28.4); the MMAs take 1.5 (KP = 48) or 3 (KP = 96).  With every
 // role in the same warps, one after the other, a tile of 1024 columns at KP =
 // 96 took 12000 clocks and one of 2048 columns at KP = 48 took 17300.
 //
@@ -265,8 +267,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
 
-// 104 registers for 416 threads: a CTA of the refinement kernel (128 threads
-// x 168) still fits on the SM beside one of this kernel
+// 104 registers: what the produced row of K = 84 components needs
 template <typename CT, int N, int G, int KC>
 __global__ void __maxnreg__(104) search_tc_kernel(const __grid_constant__ rot::SearchArgs a,
                                                   const unsigned char* __restrict__ gtab,

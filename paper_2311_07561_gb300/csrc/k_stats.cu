@@ -2,7 +2,8 @@
 //   ||P_S tau_x f||_S^2 = <(tau_x f)^2, m> - <tau_x f, m>^2 / <1, m>,
 // Algorithm 1, image block), for a binary mask given as x-runs.
 //
-// A CTA owns a 64 x 8 tile of output voxels in one z-plane.  For every mask
+// local_stats_kernel (masks that march_stats_kernel does not take): a CTA owns
+// a 64 x 8 tile of output voxels in one z-plane.  For every mask
 // plane dz it stages the rows the tile's windows touch, subtracts a reference
 // value (the input voxel at the tile centre; the variance does not change under
 // a constant shift and the shift removes the cancellation of large offsets),
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(kStatThreads) local_stats_kernel(StatsArgs a) 
 // and the plane's sum goes to the outputs z - dz that have it, kept in
 // registers until their last plane has passed.  About 140 FP64 operations per
 // voxel for a ball of radius 4, where prefix sums rebuilt for every output
-// plane took 690 (130 x 121 x 97, s = 9: 3022 us).
+// plane took 690 (130 x 121 x 97, s = 9: 3022 -> 761 us, the FP64 pipe 82% busy).
 struct MarchArgs {
     StatsArgs s;
     MarchMask m;
