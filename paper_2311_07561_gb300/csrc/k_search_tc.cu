@@ -39,9 +39,11 @@
 // role in the same warps, one after the other, a tile of 1024 columns at KP =
 // 96 took 12000 clocks and one of 2048 columns at KP = 48 took 17300.
 //
-// Waits on the mbarriers are bounded: on expiry the role leaves its loop, the
+// The roles meet on mbarriers alone (a named barrier waits without a limit),
+// and every wait on one is bounded.  On expiry the whole warp leaves its role's
+// loop (the lanes vote: the tensor-memory loads behind a wait take all 32), the
 // other roles' waits expire after it, the kernel records TTM_ERR_TIMEOUT, waits
-// once more for its MMAs and copies in flight, frees its TMEM and exits.
+// once more for its copies in flight, frees its TMEM and exits.
 #include <climits>
 
 #include <cuda_fp16.h>
@@ -98,6 +100,10 @@ constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kChunkN >> 3) << 17) | ((128
 
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase) {
     return mbar_wait_bounded(bar, phase, kMbarWaitPolls);
+}
+// the same by all lanes of a warp, with one answer for all of them
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t phase) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, phase));
 }
 
 // MMAs of one 256-point chunk whose B block (KP/8 x 32 core matrices, K-block
@@ -282,6 +288,7 @@ __global__ void __maxnreg__(104) search_tc_kernel(const __grid_constant__ rot::S
     __shared__ __align__(8) uint64_t read_s[2];      // TMEM half read by every reducing warp
     __shared__ __align__(8) uint64_t afull_s, afree_s;   // A written / read by all its MMAs
     __shared__ __align__(8) uint64_t load_s[kRing];  // grid-chunk copies
+    __shared__ __align__(8) uint64_t merge_s[kReduceWarps / 2];   // a tile's keys of warp w + 4 stored
     __shared__ uint32_t tmem_base_s;
     const int t = threadIdx.x;
     const int warp = t >> 5, lane = t & 31;
@@ -289,7 +296,7 @@ __global__ void __maxnreg__(104) search_tc_kernel(const __grid_constant__ rot::S
     int* merge = reinterpret_cast<int*>(sm + Sh::BBytes + Sh::ABytes);   // [2][KC][128]
     const uint32_t full0 = smem_u32(&full_s[0]), read0 = smem_u32(&read_s[0]);
     const uint32_t afull = smem_u32(&afull_s), afree = smem_u32(&afree_s);
-    const uint32_t load0 = smem_u32(&load_s[0]);
+    const uint32_t load0 = smem_u32(&load_s[0]), merge0 = smem_u32(&merge_s[0]);
     const uint32_t a_base = smem_u32(As), b_base = smem_u32(sm);
 
     if (warp == 0) {
@@ -305,6 +312,7 @@ __global__ void __maxnreg__(104) search_tc_kernel(const __grid_constant__ rot::S
         mbar_init(afull, kProduceWarps);
         mbar_init(afree, 1);
         for (int b = 0; b < kRing; ++b) mbar_init(load0 + 8 * b, 1);
+        for (int b = 0; b < kReduceWarps / 2; ++b) mbar_init(merge0 + 8 * b, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
@@ -343,7 +351,7 @@ __global__ void __maxnreg__(104) search_tc_kernel(const __grid_constant__ rot::S
 #pragma unroll 1
             for (int c = 0; c < kChunks; ++c) {
                 const uint32_t h = c & 1, use = (n * kChunks + c) >> 1;   // use-th chunk of half h
-                if (!mbar_wait(full0 + 8 * h, use & 1u)) { ok = false; break; }
+                if (!mbar_wait_warp(full0 + 8 * h, use & 1u)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t cols = cols0 + h * kChunkN;
                 const int low0 = 2047 - (c * kChunkN + grp * kGroupN);
@@ -371,17 +379,17 @@ __global__ void __maxnreg__(104) search_tc_kernel(const __grid_constant__ rot::S
             }
             if (!ok) break;
             // the second group hands its keys to the first (warps w and w + 4
-            // share lanes and a named barrier).  Two buffers in turn: the
-            // second group is at most two chunks ahead of the first, so it
-            // comes back to a buffer only after the first has read it.
+            // share lanes and an mbarrier).  Two buffers in turn: the second
+            // group is at most two chunks ahead of the first, so it comes back
+            // to a buffer, and to a phase, only after the first has taken it.
             int* mg = merge + (n & 1) * KC * 128 + lane_t;
             if (grp == 1) {
 #pragma unroll
                 for (int k = 0; k < KC; ++k) mg[k * 128] = top[k];
-                __threadfence_block();
-                asm volatile("bar.arrive %0, 64;\n" ::"r"(1 + (warp & 3)) : "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(merge0 + 8 * (warp & 3));
             } else {
-                asm volatile("bar.sync %0, 64;\n" ::"r"(1 + (warp & 3)) : "memory");
+                if (!mbar_wait_warp(merge0 + 8 * warp, n & 1u)) { ok = false; break; }
                 int other[KC];
 #pragma unroll
                 for (int k = 0; k < KC; ++k) other[k] = mg[k * 128];
@@ -446,7 +454,7 @@ __global__ void __maxnreg__(104) search_tc_kernel(const __grid_constant__ rot::S
                 const __half2 hh = __halves2half2(__float2half_rn(lo), __float2half_rn(hi));
                 row[j] = *reinterpret_cast<const uint32_t*>(&hh);
             }
-            if (n > 0 && !mbar_wait(afree, (n - 1) & 1u)) { ok = false; break; }
+            if (n > 0 && !mbar_wait_warp(afree, (n - 1) & 1u)) { ok = false; break; }
 #pragma unroll
             for (int kc = 0; kc < Sh::kCore; ++kc)
                 *reinterpret_cast<uint4*>(As + ((kc * 16 + (lane_t >> 3)) * 8 + (lane_t & 7)) * 16) =

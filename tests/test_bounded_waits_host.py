@@ -1,0 +1,45 @@
+"""The roles of the tensor-core search meet in waits that end (no GPU).
+
+The kernel's warps take three roles (reduce, produce, issue) that leave their
+loops when a bounded wait runs out.  From there on no other role may wait for
+them without a limit, and no lane of a warp may go on alone into the
+tensor-memory loads and warp barriers that take all 32.  That is a property of
+the source, and it is read from there: making a wait run out inside the kernel
+would need a GPU that stalls for a second.
+"""
+
+import os
+import re
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SEARCH = os.path.join(ROOT, "paper_2311_07561_gb300", "csrc", "k_search_tc.cu")
+
+
+def _code():
+    text = open(SEARCH).read()
+    return re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+
+
+def _roles():
+    """Source of the whole-warp roles (reduce, produce) and of the issuing thread."""
+    text = _code()
+    begin = text.index("if (warp < kReduceWarps) {")
+    issue = text.index("if (lane == 0 && mine > 0) {", begin)
+    end = text.index("__syncthreads_and(ok)", issue)
+    return text[begin:issue], text[issue:end]
+
+
+def test_roles_wait_on_mbarriers_only():
+    warps, issue = _roles()
+    unlimited = re.compile(r"\bbar\.(?:sync|arrive|red)|\bbarrier\.|__syncthreads|__nanosleep")
+    assert not unlimited.findall(warps)
+    assert not unlimited.findall(issue)
+
+
+def test_whole_warps_leave_together():
+    warps, issue = _roles()
+    assert not re.findall(r"\bmbar_wait(?:_bounded)?\s*\(", warps), "a wait without a vote"
+    assert re.findall(r"\bmbar_wait_warp\s*\(", warps)
+    assert not re.findall(r"\bmbar_wait_warp\s*\(", issue), "a vote by one lane"
+    vote = re.search(r"bool mbar_wait_warp\([^)]*\)\s*\{([^}]*)\}", _code()).group(1)
+    assert "__all_sync(0xffffffffu, mbar_wait(" in vote
