@@ -43,7 +43,7 @@
 // and every wait on one is bounded.  On expiry the whole warp leaves its role's
 // loop (the lanes vote: the tensor-memory loads behind a wait take all 32), the
 // other roles' waits expire after it, the kernel records TTM_ERR_TIMEOUT, waits
-// once more for its copies in flight, frees its TMEM and exits.
+// once more for its MMAs and copies in flight, frees its TMEM and exits.
 #include <climits>
 
 #include <cuda_fp16.h>
@@ -504,14 +504,14 @@ __global__ void __maxnreg__(104) search_tc_kernel(const __grid_constant__ rot::S
                 }
             }
         }
-        if (!ok) {
-            // MMAs and copies in flight finish before the memory is released
-            for (uint32_t hh = 0; hh < 2; ++hh)
-                if ((pending >> hh) & 1u) {
-                    const uint32_t last = q > 0 && ((q - 1) & 1u) == hh ? q - 1 : q - 2;
-                    mbar_wait(full0 + 8 * hh, (last >> 1) & 1u);
-                }
-        }
+        // MMAs and copies in flight finish before the memory is released: also
+        // when every chunk was issued, as a reducing warp that gave up on the
+        // last of them does not wait for it
+        for (uint32_t hh = 0; hh < 2; ++hh)
+            if ((pending >> hh) & 1u) {
+                const uint32_t last = q > 0 && ((q - 1) & 1u) == hh ? q - 1 : q - 2;
+                mbar_wait(full0 + 8 * hh, (last >> 1) & 1u);
+            }
         for (uint32_t b = 0; b < (uint32_t)kRing; ++b)
             if ((loading >> b) & 1u) {
                 uint32_t lq = b;                  // the buffer's latest copy

@@ -43,3 +43,14 @@ def test_whole_warps_leave_together():
     assert not re.findall(r"\bmbar_wait_warp\s*\(", issue), "a vote by one lane"
     vote = re.search(r"bool mbar_wait_warp\([^)]*\)\s*\{([^}]*)\}", _code()).group(1)
     assert "__all_sync(0xffffffffu, mbar_wait(" in vote
+
+
+def test_issuer_drains_its_mmas_on_every_path():
+    """A reducing warp may give up after the last chunk was issued: the issuing
+    thread then leaves its loop without a fault of its own, and still has to see
+    the MMAs done before the kernel frees the tensor memory they write."""
+    _, issue = _roles()
+    drain = issue[issue.index("for (uint32_t hh = 0"):]
+    before = issue[:issue.index("for (uint32_t hh = 0")].rstrip()
+    assert "mbar_wait(full0 + 8 * hh" in drain
+    assert not re.search(r"if\s*\([^)]*ok[^)]*\)\s*\{$", before), "drained only after a wait of its own ran out"
