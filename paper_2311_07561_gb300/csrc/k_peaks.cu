@@ -5,7 +5,8 @@
 //
 // Three passes: the voxels above the threshold that are the largest of their
 // 3^3 cube (a few in a hundred) with the maxima of 4^3 cells, then those that
-// no cell inside their cube beats, then the voxels of the cubes that are left.
+// no cell inside their cube beats, then the voxels of the cubes that are left
+// (up to radius 4 the cubes at once).
 // Few loads per voxel are needed either way, so the passes are bound by L1/L2
 // and latency, not by the (2r+1) loads per axis of a separable maximum (256^3,
 // r = 12: 1559 us).
@@ -126,7 +127,7 @@ __device__ __forceinline__ void emit_peak(int v, const float* __restrict__ score
     list[slot] = rec;
 }
 
-// radius 0: every candidate is a peak
+// radius 0 and 1: every candidate is a peak
 __global__ void __launch_bounds__(256) peak_all_kernel(
     const float* __restrict__ score, const float* __restrict__ quat, const float* __restrict__ lam,
     const int* __restrict__ cand, const int* __restrict__ n_cand, PeakRec* __restrict__ list, int cap,
@@ -177,6 +178,45 @@ __global__ void __launch_bounds__(256) peak_cells_kernel(
             }
         }
         if (!beaten) left[atomicAdd(n_left, 1)] = v;
+    }
+}
+
+// Radius 2 to 4: one warp per candidate.  The cube has 125 to 729 voxels and
+// hardly a whole cell, and a few voxels in a hundred are candidates: cells that
+// turn almost none of them away, then a CTA with its block-wide votes for each,
+// took longer than the separable maximum these passes replace (256 x 251 x 259
+// of noise, peak kernels: r = 2 509 us before them, 1262 with a CTA each, 316
+// now; r = 3 554, 647, 356; r = 4 613, 431, 396; at r = 5 the cells pay: 260
+// against 438).
+constexpr int kWarpRadius = 4;
+
+__global__ void __launch_bounds__(256) peak_warp_kernel(
+    const float* __restrict__ score, const float* __restrict__ quat, const float* __restrict__ lam,
+    int X, int Y, int Z, int r, const int* __restrict__ cand, const int* __restrict__ n_cand,
+    PeakRec* __restrict__ list, int cap, int* __restrict__ count) {
+    const int n = *n_cand, lane = threadIdx.x & 31;
+    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += gridDim.x * 8) {
+        const int v = __ldg(cand + i);
+        const float s = __ldg(score + v);
+        const int row = v / X, x = v - row * X, z = row / Y, y = row - z * Y;
+        const int xa = max(x - r, 0), w = min(x + r, X - 1) - xa + 1;
+        const int ya = max(y - r, 0), h = min(y + r, Y - 1) - ya + 1;
+        const int za = max(z - r, 0), d = min(z + r, Z - 1) - za + 1;
+        bool beaten = false;
+        for (int e0 = 0; e0 < w * h * d && !beaten; e0 += 128) {    // four loads in flight
+            bool hit = false;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int e = e0 + 32 * j + lane;
+                if (e >= w * h * d) break;
+                const int rr = e / w, rz = rr / h;
+                const int o_at = ((za + rz) * Y + ya + (rr - rz * h)) * X + xa + (e - rr * w);
+                const float o = __ldg(score + o_at);
+                hit = hit || o > s || (o == s && o_at < v);
+            }
+            beaten = __any_sync(0xffffffffu, hit);
+        }
+        if (!beaten && lane == 0) emit_peak(v, score, quat, lam, list, cap, count);
     }
 }
 
@@ -281,8 +321,13 @@ ttm_status launch_peak_candidates_full(const float* score, const float* quat, co
     if (grid.y > 65535u || grid.z > 65535u) return TTM_ERR_UNSUPPORTED;
     peak_candidates_kernel<<<grid, 256, 0, st>>>(score, X, Y, Z, radius, thr, cand, n_cand, cells);
     TTM_TRY(after_launch(cnt));
-    if (radius == 0) {
+    if (radius <= 1) {                                   // the first pass took the whole cube
         peak_all_kernel<<<152 * 8, 256, 0, st>>>(score, quat, lam, cand, n_cand, recs, cap, d_count);
+        return after_launch(cnt);
+    }
+    if (radius <= kWarpRadius) {
+        peak_warp_kernel<<<152 * 8, 256, 0, st>>>(score, quat, lam, X, Y, Z, radius, cand, n_cand, recs, cap,
+                                                  d_count);
         return after_launch(cnt);
     }
     peak_cells_kernel<<<152 * 8, 256, 0, st>>>(score, X, Y, Z, radius, cand, n_cand, cells, left, n_left);

@@ -219,3 +219,24 @@ def test_classical_long_z(ttm, depth, s, n_rot):
     assert np.abs(best - best_o).max() <= TOL
     zi, yi, xi = np.nonzero(keep)
     assert np.all(c[arg[zi, yi, xi], zi, yi, xi] >= best_o[zi, yi, xi] - TOL)
+
+
+@pytest.mark.parametrize("shape", [(6, 5, 7), (33, 40, 70), (19, 9, 130)])
+def test_peaks_of_small_cubes(ttm, shape):
+    """Radii up to the last one that scans its cubes without cells, and the
+    next: few levels, so that ties decide, and a map with many peaks."""
+    Z, Y, X = shape
+    rng = np.random.default_rng(X)
+    t = synth.blob_template(5, 3, seed=1)
+    comp, desc = ttm.build_template(t, synth.ball_mask(5, 2), 2,
+                                    synth.super_fibonacci_quaternions(10).astype(np.float32))
+    m = ttm.Matcher([(comp, desc, synth.ball_mask(5, 2))], [((X, Y, Z), 0)])
+    quat = np.zeros(shape + (4,), dtype=np.float32)
+    for levels in (2, 10 ** 6):
+        score = (np.floor(rng.random(shape) * levels) / levels + 0.25).astype(np.float32)
+        for radius in (1, 2, 3, 4, 5):
+            got = ttm.ttm_extract_peaks(m.plan, 0, _cuda(score), _cuda(quat), _cuda(score), 0.2,
+                                        radius, score.size, m.ws)
+            expect = o.extract_peaks(score.astype(np.float64), 0.2, radius, score.size)
+            assert np.array_equal((got["z"].astype(np.int64) * Y + got["y"]) * X + got["x"], expect)
+    m.close()
