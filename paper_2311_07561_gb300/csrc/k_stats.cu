@@ -2,13 +2,13 @@
 //   ||P_S tau_x f||_S^2 = <(tau_x f)^2, m> - <tau_x f, m>^2 / <1, m>,
 // Algorithm 1, image block), for a binary mask given as x-runs.
 //
-// local_stats_kernel (masks that march_stats_kernel does not take): a CTA owns
-// a 64 x 8 tile of output voxels in one z-plane.  For every mask
-// plane dz it stages the rows the tile's windows touch, subtracts a reference
-// value (the input voxel at the tile centre; the variance does not change under
-// a constant shift and the shift removes the cancellation of large offsets),
-// and builds exclusive prefix sums of (f - mu) and (f - mu)^2 along x in
-// shared memory.  Each x-run of the mask then costs two prefix lookups per
+// local_stats_kernel (masks that march_stats_kernel does not take, and volumes
+// too small for it): a CTA owns a 64 x 8 tile of output voxels in one z-plane.
+// For every mask plane dz it stages the rows the tile's windows touch, subtracts
+// a reference value (the input voxel at the tile centre; the variance does not
+// change under a constant shift and the shift removes the cancellation of large
+// offsets), and builds exclusive prefix sums of (f - mu) and (f - mu)^2 along x
+// in shared memory.  Each x-run of the mask then costs two prefix lookups per
 // statistic.  The prefix sums and S1, S2 are FP64: a difference of two prefix
 // sums cancels whatever the row holds before the run, which in FP32 loses a
 // quiet run next to a bright one.  V = S2 - S1^2/m_sum is formed in FP64.
@@ -311,6 +311,40 @@ __global__ void __launch_bounds__(256) exterior_zero_kernel(float* __restrict__ 
     }
 }
 
+// Output planes per CTA of the march, and whether it beats local_stats_kernel.
+// A CTA passes planes + ndz - 1 input planes; CTAs beyond one per SM wait for
+// their turn at the FP64 pipe (two on an SM take 1.8 times one).  At the least
+// cost by that count a plane of the march takes (ndz + 3) / 8 times one of
+// local_stats_kernel, which passes ndz planes for every output plane: its windows
+// are a chain of additions, and in a volume too small to fill the SMs
+// nothing hides it.  ms, s = 9: 20^3 and 30^3 0.133 there, marching 0.174 at
+// best; 40 x 41 x 37 0.226, 0.175; 64^3 0.428, 0.259; 130 x 121 x 97 3.06,
+// 0.79.  s = 15: 40 x 41 x 37 0.527, 0.580; 64^3 1.03, 0.73.  (With 8 planes
+// and more per CTA whatever the volume, 20^3 took 0.287 and 0.757.)
+struct MarchSplit {
+    int planes;
+    bool pays;
+};
+
+MarchSplit march_split(int X, int Y, int Z, int gx, int gy, int nz, int ndz) {
+    auto turns = [](double ctas) {
+        const double t = ceil(ctas / 152.0);
+        return t < 1.1 ? 1.1 : t;
+    };
+    MarchSplit best{1, true};
+    double least = 0.0;
+    for (int n = 1; n <= 64 && n <= nz; ++n) {
+        const double parts = (double)((nz + n - 1) / n);
+        const double cost = (n + ndz - 1) * turns((double)gx * gy * parts);
+        if (parts > 65535.0 || (least > 0.0 && cost >= least)) continue;
+        least = cost;
+        best.planes = n;
+    }
+    const double other = ndz * turns((double)((X + kTX - 1) / kTX) * ((Y + kTY - 1) / kTY) * Z);
+    best.pays = Z > 65535 || least * (ndz + 3) / 8.0 <= other;
+    return best;
+}
+
 template <int NDZ>
 ttm_status march_launch(const MarchArgs& a, dim3 grid, size_t smem, int ndz, cudaStream_t st) {
     if constexpr (NDZ > 1) {
@@ -421,23 +455,18 @@ ttm_status launch_local_stats(const float* f, int X, int Y, int Z, const Templat
     a.moments = d_moments;
     const VoxBox box = interior_box(X, Y, Z, T.desc.s);
     if (T.march.n_win > 0 && box.count() > 0) {
-        // every output's planes lie in the volume (a mask reaches at most its
-        // box).  Planes per CTA: fewer cost more halo planes, more leave SMs
-        // idle; at most two CTAs per SM (FP64 sets the pace, so a third on some
-        // SMs is half the time again), at least 8 planes
+        // every output's planes lie in the volume (a mask reaches at most its box)
         MarchArgs m;
         m.s = a; m.m = T.march; m.runs = T.d_march_runs;
         m.x0 = box.x0; m.y0 = box.y0; m.z0 = box.z0; m.z1 = box.z0 + (int)box.nz - 1;
         const int gx = ((int)box.nx + kMarchX - 1) / kMarchX, gy = ((int)box.ny + kMarchY - 1) / kMarchY;
-        const int want = 304 / (gx * gy) > 1 ? 304 / (gx * gy) : 1;
-        int nzc = ((int)box.nz + want - 1) / want;
-        nzc = nzc < 8 ? 8 : nzc > 64 ? 64 : nzc;
-        m.nzc = nzc;
         const int ndz = T.dz_max - T.dz_min + 1;
         const int rows = kMarchY + (T.dy_max - T.dy_min), width = kMarchX + (T.x_max - T.x_min);
         const size_t smem = (size_t)rows * (T.march.n_win * kMarchX * 16 + width * 8);
-        const dim3 grid(gx, gy, ((int)box.nz + nzc - 1) / nzc);
-        if (gy <= 65535) {
+        const MarchSplit split = march_split(X, Y, Z, gx, gy, (int)box.nz, ndz);
+        m.nzc = split.planes;
+        const dim3 grid(gx, gy, ((int)box.nz + m.nzc - 1) / m.nzc);
+        if (gy <= 65535 && split.pays) {
             exterior_zero_kernel<<<152 * 8, 256, 0, st>>>(w, X, Y, Z, T.desc.s);
             TTM_TRY(after_launch(cnt));
             TTM_TRY(march_launch<kMarchDz>(m, grid, smem, ndz, st));

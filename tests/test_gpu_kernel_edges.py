@@ -240,3 +240,21 @@ def test_peaks_of_small_cubes(ttm, shape):
             expect = o.extract_peaks(score.astype(np.float64), 0.2, radius, score.size)
             assert np.array_equal((got["z"].astype(np.int64) * Y + got["y"]) * X + got["x"], expect)
     m.close()
+
+
+@pytest.mark.parametrize("s,shape", [(5, (21, 20, 22)), (7, (33, 41, 66)), (9, (20, 21, 22)), (9, (37, 41, 40)),
+                                     (11, (30, 43, 90)), (13, (52, 48, 47)), (15, (37, 41, 40)),
+                                     (15, (64, 60, 62))])
+def test_direct_statistics_of_both_forms(ttm, s, shape):
+    """Volumes on both sides of the line between marching and one plane at a
+    time, the marching ones with one to several planes per block."""
+    rng = np.random.default_rng(s)
+    mask = _mask("ball", s)
+    volume = (rng.normal(size=shape) + 3.0).astype(np.float32)
+    q = synth.super_fibonacci_quaternions(8).astype(np.float32)
+    comp, desc = ttm.build_template(rng.normal(size=(s, s, s)).astype(np.float32), mask, 2, q)
+    res, _ = _maps(ttm, volume, comp, desc, mask, path=ttm.TTM_PATH_DIRECT)
+    w_o = o.local_stats_direct(volume, mask)[2]
+    nz = w_o > 0
+    assert np.array_equal(res["w"] > 0, nz)
+    assert (np.abs(res["w"][nz] - w_o[nz]) / w_o[nz]).max() <= 1e-5
