@@ -236,10 +236,12 @@ __global__ void __launch_bounds__(kMarchX * kMarchY) march_stats_kernel(const __
         sh[1] = 1e-6 * a.s.mask_sum * var_f;
     }
     // reference value near the middle of the tile (the variance does not
-    // change under a shift, which removes the cancellation of large offsets)
-    const double mu = __ldg(a.s.f + ((size_t)min((z0 + z1) / 2, a.s.Z - 1) * a.s.Y +
+    // change under a shift, which removes the cancellation of large offsets);
+    // one that is not finite would take every window of the tile with it
+    const float ref = __ldg(a.s.f + ((size_t)min((z0 + z1) / 2, a.s.Z - 1) * a.s.Y +
                                      min(y0 + kMarchY / 2, a.s.Y - 1)) * a.s.X +
                             min(x0 + kMarchX / 2, a.s.X - 1));
+    const double mu = isfinite(ref) ? (double)ref : 0.0;
     double s1[NDZ], s2[NDZ];                 // slot k: output plane zz - dz_min - k
 #pragma unroll
     for (int k = 0; k < NDZ; ++k) s1[k] = s2[k] = 0.0;

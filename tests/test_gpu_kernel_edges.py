@@ -258,3 +258,34 @@ def test_direct_statistics_of_both_forms(ttm, s, shape):
     nz = w_o > 0
     assert np.array_equal(res["w"] > 0, nz)
     assert (np.abs(res["w"][nz] - w_o[nz]) / w_o[nz]).max() <= 1e-5
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_direct_statistics_beside_values_that_are_not_finite(ttm, value):
+    """Columns of such values at a block's reference voxel: the windows that
+    hold one have no w, every other window has its own."""
+    s, shape = 5, (30, 44, 70)
+    mask = _mask("ball", s)
+    rng = np.random.default_rng(12)
+    volume = (rng.normal(size=shape) + 3.0).astype(np.float32)
+    q = synth.super_fibonacci_quaternions(8).astype(np.float32)
+    comp, desc = ttm.build_template(rng.normal(size=(s, s, s)).astype(np.float32), mask, 2, q)
+    touched = np.zeros(shape, bool)
+    disc = mask.any(axis=0)
+    w_o = o.local_stats_direct(volume, mask)[2]
+    for x, y in ((18, 6), (18, 14), (50, 30)):
+        volume[:, y, x] = value
+        for dy, dx in np.argwhere(disc) - s // 2:
+            touched[:, y - dy, x - dx] = True
+    import torch
+    po = ttm.PlanOpts()
+    po.path = ttm.TTM_PATH_DIRECT
+    m = ttm.Matcher([(comp, desc, mask)], [(shape[::-1], 0)], opts=po)
+    ttm.ttm_local_stats(m.plan, [_cuda(volume)], m.w, m.ws)
+    torch.cuda.synchronize()
+    w = m.w[0].cpu().numpy()
+    m.close()
+    keep = (w_o > 0) & ~touched
+    assert keep.sum() > 20000
+    assert np.all(w[touched] == 0)
+    assert (np.abs(w[keep] - w_o[keep]) / w_o[keep]).max() <= 1e-5
