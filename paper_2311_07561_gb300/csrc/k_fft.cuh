@@ -548,7 +548,7 @@ __device__ __forceinline__ void stages_io(const Src& src, float2* a, float2* b, 
 // A tile is NB consecutive half-spectrum rows (contiguous in memory) of one z
 // plane of one batch item; only the planes z0..z1 and the rows y0..y1 of the
 // keep box are visited (tiles start at multiples of NB rows, so every tile is
-// one aligned bulk copy).  Each CTA walks tiles with a stride of gridDim.x;
+// one aligned bulk copy, or one for each padded row).  Each CTA walks tiles with a stride of gridDim.x;
 // the next NST - 1 tiles are in flight in a ring of staging buffers (bulk
 // copies completing on one mbarrier each) while the current one is
 // transformed.  The first stage reads the staged rows with the Hermitian
@@ -559,8 +559,20 @@ __device__ __forceinline__ void stages_io(const Src& src, float2* a, float2* b, 
 template <int L>
 constexpr int c2r_stages_buffers() { return n_stages(L) >= 3 ? 2 : 1; }
 
+// Staged rows: as they are in memory where they are not padded (one bulk copy
+// a tile), else each by a copy of its own without the padding: the lanes of a
+// warp read neighbouring rows, and a pitch of 72 samples (128 points) puts eight
+// of them on the same banks, one of 66 (FP32) or 68 (bf16) none or two.  y and x
+// passes of 35 FP32 components, 126 x 126 x 480: 1203 us with the tile as it
+// is, 979 now (971 before the spectra's rows were padded).
 template <int L, typename PS>
-constexpr uint32_t c2r_tile_bytes() { return (uint32_t)(rows_nb<L>() * spec_pitch(L) * sizeof(PS)); }
+constexpr uint32_t c2r_row_bytes() {
+    return (uint32_t)(spec_pitch(L) == L / 2 + 1 ? (L / 2 + 1) * sizeof(PS)
+                                                 : ((L / 2 + 1) * sizeof(PS) + 15) / 16 * 16);
+}
+
+template <int L, typename PS>
+constexpr uint32_t c2r_tile_bytes() { return rows_nb<L>() * c2r_row_bytes<L, PS>(); }
 
 template <int L>
 constexpr size_t c2r_fft_bytes() {
@@ -584,10 +596,12 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-__device__ __forceinline__ void bulk_to_smem(uint32_t dst, const void* src, uint32_t bytes,
-                                             uint32_t bar) {
+// arms the barrier for `bytes`; copies of that many bytes in all complete on it
+__device__ __forceinline__ void bulk_expect(uint32_t bytes, uint32_t bar) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
                  : "memory");
+}
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
         ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
@@ -640,6 +654,27 @@ __global__ void __launch_bounds__(kFftThreads) rows_c2r_t(const PS* __restrict__
         return in + ((item * (size_t)g.Zp + (size_t)z) * (size_t)g.Yp + (size_t)y_start) * spec_pitch(L);
     };
     const uint32_t sbase = smem_addr(smraw);
+    constexpr bool ROWS = spec_pitch(L) != XH;      // a copy per row, by the lanes of the first warp
+    constexpr int SROW = (int)(c2r_row_bytes<L, PS>() / sizeof(PS));
+    static_assert(!ROWS || SROW * sizeof(PS) % 32 == 16, "rows an odd number of 16-byte units apart");
+    static_assert(!ROWS || (NB <= 32 && spec_pitch(L) * sizeof(PS) % 16 == 0), "rows on 16-byte boundaries");
+    // tile t into staging buffer q (by the first warp, or its first thread)
+    auto fetch = [&](size_t t, int q) {
+        int ys, z;
+        size_t item;
+        const PS* src = tile_src(t, ys, item, z);
+        const uint32_t dst = sbase + (uint32_t)q * TILE, bar = smem_addr(&bars[q]);
+        if constexpr (ROWS) {
+            constexpr uint32_t RB = c2r_row_bytes<L, PS>();
+            if (threadIdx.x == 0) bulk_expect(TILE, bar);
+            __syncwarp();
+            if (threadIdx.x < NB) bulk_copy(dst + threadIdx.x * RB, src + threadIdx.x * spec_pitch(L), RB, bar);
+        } else {
+            bulk_expect(TILE, bar);
+            bulk_copy(dst, src, TILE, bar);
+        }
+    };
+    const bool fetches = threadIdx.x < (ROWS ? 32 : 1);
     if (threadIdx.x == 0) {
         for (int q = 0; q < NST; ++q)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(&bars[q])) : "memory");
@@ -648,15 +683,12 @@ __global__ void __launch_bounds__(kFftThreads) rows_c2r_t(const PS* __restrict__
     }
     __syncthreads();
     if ((size_t)blockIdx.x >= ntiles) return;
-    uint32_t pending = 0u;                   // thread 0: buffers with a copy in flight
-    if (threadIdx.x == 0) {
+    uint32_t pending = 0u;                   // buffers with a copy in flight
+    if (fetches) {
         for (int q = 0; q < NST - 1; ++q) {
             const size_t t = blockIdx.x + (size_t)q * gridDim.x;
             if (t >= ntiles) break;
-            int ys, z;
-            size_t item;
-            bulk_to_smem(sbase + (uint32_t)q * TILE, tile_src(t, ys, item, z), TILE,
-                         smem_addr(&bars[q]));
+            fetch(t, q);
             pending |= 1u << q;
         }
     }
@@ -664,15 +696,12 @@ __global__ void __launch_bounds__(kFftThreads) rows_c2r_t(const PS* __restrict__
     int it = 0;
     for (size_t tile = blockIdx.x; tile < ntiles; ++it, tile += gridDim.x) {
         const int buf = it % NST;
-        if (threadIdx.x == 0) {
+        if (fetches) {
             const size_t ahead = tile + (size_t)(NST - 1) * gridDim.x;
             if (ahead < ntiles) {
                 const int nb = (it + NST - 1) % NST;
-                int ys, z;
-                size_t item;
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                bulk_to_smem(sbase + (uint32_t)nb * TILE, tile_src(ahead, ys, item, z), TILE,
-                             smem_addr(&bars[nb]));
+                fetch(ahead, nb);
                 pending |= 1u << nb;
             }
         }
@@ -699,8 +728,8 @@ __global__ void __launch_bounds__(kFftThreads) rows_c2r_t(const PS* __restrict__
         const int xk0 = keep.x0, xk1 = min(keep.x1, X - 1);
         stages_io<L, 0, NB, PITCH, +1>(
             [S](int x, int line) {
-                if (x < XH) return ldc(S + line * spec_pitch(L) + x);
-                const float2 c = ldc(S + line * spec_pitch(L) + (L - x));
+                if (x < XH) return ldc(S + line * SROW + x);
+                const float2 c = ldc(S + line * SROW + (L - x));
                 return make_float2(c.x, -c.y);
             },
             a, b,
