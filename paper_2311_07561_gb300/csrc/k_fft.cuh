@@ -958,8 +958,7 @@ cudaError_t run_rows_c2r(const PS* prod, int X, int Y, int Z, FftGeom g, RT* cor
         (void)status;                       // no device-side waits in this pass
         kern<<<grid, kRowThreads, smem, st>>>(prod, X, Y, Z, g, corr, K, tw, keep);
         return cudaGetLastError();
-    }
-    if constexpr (c2r_half<L>() && !rows_packed<L>()) {
+    } else if constexpr (c2r_half<L>()) {
         constexpr int L1 = RowSplit<L / 2>::L1, L2 = RowSplit<L / 2>::L2;
         constexpr int NR = kTwoThreads / L1 * c2r_groups<L1, L2, PS>();   // rows per tile
         constexpr size_t smem = c2r_half_smem<L1, L2, PS>();
@@ -975,26 +974,27 @@ cudaError_t run_rows_c2r(const PS* prod, int X, int Y, int Z, FftGeom g, RT* cor
         (void)status;                       // no device-side waits in this pass
         kern<<<grid, kTwoThreads, smem, st>>>(prod, X, Y, Z, g, corr, K, tw, keep);
         return cudaGetLastError();
+    } else {
+        constexpr int NB = rows_nb<L>();
+        constexpr size_t smem = c2r_smem<L, PS>();
+        cudaError_t e = cudaFuncSetAttribute(rows_c2r_t<L, PS, RT>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        int sms = 0, per_sm = 0;
+        if ((e = sm_count(&sms)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rows_c2r_t<L, PS, RT>,
+                                                               kFftThreads, smem)) != cudaSuccess)
+            return e;
+        if (keep.z1 < keep.z0 || keep.y1 < keep.y0 || keep.x1 < keep.x0) return cudaSuccess;
+        const int nty = (keep.y1 - (keep.y0 & ~(NB - 1))) / NB + 1;
+        const size_t ntiles = (size_t)K * (keep.z1 - keep.z0 + 1) * nty;
+        const size_t cap = (size_t)sms * (per_sm > 0 ? per_sm : 1);
+        const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
+        if (grid == 0) return cudaSuccess;
+        rows_c2r_t<L, PS, RT><<<grid, kFftThreads, smem, st>>>(prod, X, Y, Z, g, corr, K, tw, status,
+                                                              keep);
+        return cudaGetLastError();
     }
-    constexpr int NB = rows_nb<L>();
-    constexpr size_t smem = c2r_smem<L, PS>();
-    cudaError_t e = cudaFuncSetAttribute(rows_c2r_t<L, PS, RT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int sms = 0, per_sm = 0;
-    if ((e = sm_count(&sms)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rows_c2r_t<L, PS, RT>,
-                                                           kFftThreads, smem)) != cudaSuccess)
-        return e;
-    if (keep.z1 < keep.z0 || keep.y1 < keep.y0 || keep.x1 < keep.x0) return cudaSuccess;
-    const int nty = (keep.y1 - (keep.y0 & ~(NB - 1))) / NB + 1;
-    const size_t ntiles = (size_t)K * (keep.z1 - keep.z0 + 1) * nty;
-    const size_t cap = (size_t)sms * (per_sm > 0 ? per_sm : 1);
-    const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
-    if (grid == 0) return cudaSuccess;
-    rows_c2r_t<L, PS, RT><<<grid, kFftThreads, smem, st>>>(prod, X, Y, Z, g, corr, K, tw, status,
-                                                          keep);
-    return cudaGetLastError();
 }
 
 }  // namespace fftk
@@ -1040,16 +1040,17 @@ cudaError_t FftLen<L>::rows_r2c(const float* f, int X, int Y, int Z, FftGeom g, 
         if (grid == 0) return cudaSuccess;
         kern<<<grid, fftk::kTwoThreads, smem, st>>>(f, X, Y, Z, g, spec, tw, mode, moments, box);
         return cudaGetLastError();
+    } else {
+        constexpr int NB = fftk::rows_nb<L>();
+        const size_t smem = (size_t)2 * L * (NB + 1) * sizeof(float2);
+        cudaError_t e = cudaFuncSetAttribute(fftk::rows_r2c_t<L>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const long long nrows = box.s ? (long long)box.n * box.s * box.s : (long long)g.Yp * g.Zp;
+        fftk::rows_r2c_t<L><<<(unsigned)((nrows + NB - 1) / NB), fftk::kFftThreads, smem, st>>>(
+            f, X, Y, Z, g, spec, tw, mode, moments, box);
+        return cudaGetLastError();
     }
-    constexpr int NB = fftk::rows_nb<L>();
-    const size_t smem = (size_t)2 * L * (NB + 1) * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(fftk::rows_r2c_t<L>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const long long nrows = box.s ? (long long)box.n * box.s * box.s : (long long)g.Yp * g.Zp;
-    fftk::rows_r2c_t<L><<<(unsigned)((nrows + NB - 1) / NB), fftk::kFftThreads, smem, st>>>(
-        f, X, Y, Z, g, spec, tw, mode, moments, box);
-    return cudaGetLastError();
 }
 
 template <int L>
