@@ -714,8 +714,6 @@ __global__ void __launch_bounds__(kFftThreads) rows_c2r_t(const PS* __restrict__
                 ? (long long)(item * ((size_t)X * Y * Z) + ((size_t)z * Y + y) * X) : -1;
         }
         const bool ok = bar_wait(smem_addr(&bars[buf]), (phase >> buf) & 1u);
-        phase ^= 1u << buf;
-        if (threadIdx.x == 0) pending &= ~(1u << buf);
         if (__syncthreads_or(!ok)) {
             if (threadIdx.x == 0) {
                 atomicExch(status, TTM_ERR_TIMEOUT);
@@ -724,6 +722,8 @@ __global__ void __launch_bounds__(kFftThreads) rows_c2r_t(const PS* __restrict__
             }
             return;
         }
+        phase ^= 1u << buf;                  // (one that was given up on is still in flight)
+        pending &= ~(1u << buf);
         const PS* S = reinterpret_cast<const PS*>(smraw + (size_t)buf * TILE);
         const int xk0 = keep.x0, xk1 = min(keep.x1, X - 1);
         stages_io<L, 0, NB, PITCH, +1>(

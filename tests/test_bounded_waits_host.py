@@ -54,3 +54,17 @@ def test_issuer_drains_its_mmas_on_every_path():
     before = issue[:issue.index("for (uint32_t hh = 0")].rstrip()
     assert "mbar_wait(full0 + 8 * hh" in drain
     assert not re.search(r"if\s*\([^)]*ok[^)]*\)\s*\{$", before), "drained only after a wait of its own ran out"
+
+
+def test_row_pass_counts_a_copy_it_gave_up_on_as_in_flight():
+    """The inverse row pass waits once more for its copies in flight before it
+    returns with TTM_ERR_TIMEOUT; the one whose wait ran out is among them."""
+    text = open(os.path.join(os.path.dirname(SEARCH), "k_fft.cuh")).read()
+    text = re.sub(r"//[^\n]*", "", text)
+    kernel = text[text.index("rows_c2r_t(const PS*"):]
+    kernel = kernel[:kernel.index("stages_io<")]
+    wait = kernel.index("const bool ok = bar_wait(")
+    left = kernel.index("return;", wait)
+    assert "bar_wait(" in kernel[wait + 30:left], "no second wait"
+    assert not re.search(r"pending &=|phase \^=", kernel[wait:left])
+    assert re.search(r"pending &= ~", kernel[left:]) and re.search(r"phase \^=", kernel[left:])
