@@ -42,9 +42,14 @@ __global__ void __launch_bounds__(256) peak_candidates_kernel(
     __shared__ int n_found, base_s;
     __shared__ float part[8][32 / kCell][kWalk / kCell];      // [y][cell x][cell z]
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int x = blockIdx.x * 32 + lane;
-    const int y = blockIdx.y * 8 + warp;
-    const int z0 = blockIdx.z * kWalk, z1 = min(z0 + kWalk, Z);
+    // block (bx, by, bz) of a one-dimensional grid: y and z may be longer than
+    // a grid's second and third extent
+    const unsigned nbx = (unsigned)(X + 31) / 32, nby = (unsigned)(Y + 7) / 8;
+    const int bx = (int)(blockIdx.x % nbx), by = (int)(blockIdx.x / nbx % nby),
+              bz = (int)(blockIdx.x / nbx / nby);
+    const int x = bx * 32 + lane;
+    const int y = by * 8 + warp;
+    const int z0 = bz * kWalk, z1 = min(z0 + kWalk, Z);
     const size_t plane = (size_t)X * Y;
     const bool in = x < X && y < Y;
     const int xc = min(x, X - 1), yc = min(y, Y - 1);
@@ -104,8 +109,7 @@ __global__ void __launch_bounds__(256) peak_candidates_kernel(
         float m = part[cy * kCell][cx][cz];
 #pragma unroll
         for (int k = 1; k < kCell; ++k) m = fmaxf(m, part[cy * kCell + k][cx][cz]);
-        const int gx = blockIdx.x * (32 / kCell) + cx, gy = blockIdx.y * 2 + cy,
-                  gz = blockIdx.z * (kWalk / kCell) + cz;
+        const int gx = bx * (32 / kCell) + cx, gy = by * 2 + cy, gz = bz * (kWalk / kCell) + cz;
         if (gx < CX && gy < CY && gz < CZ) cells[((size_t)gz * CY + gy) * CX + gx] = m;
     }
     __syncthreads();
@@ -185,9 +189,9 @@ __global__ void __launch_bounds__(256) peak_cells_kernel(
 // hardly a whole cell, and a few voxels in a hundred are candidates: cells that
 // turn almost none of them away, then a CTA with its block-wide votes for each,
 // took longer than the separable maximum these passes replace (256 x 251 x 259
-// of noise, peak kernels: r = 2 509 us before them, 1262 with a CTA each, 316
-// now; r = 3 554, 647, 356; r = 4 613, 431, 396; at r = 5 the cells pay: 260
-// against 438).
+// of noise, peak kernels: r = 1 465 us before them, 1552 with a CTA each, 123
+// now; r = 2 515, 1255, 316; r = 3 553, 644, 361; r = 4 621, 433, 393; at r = 5
+// the cells pay: 260 against 438).
 constexpr int kWarpRadius = 4;
 
 __global__ void __launch_bounds__(256) peak_warp_kernel(
@@ -317,8 +321,8 @@ ttm_status launch_peak_candidates_full(const float* score, const float* quat, co
     int* n_left = d_count + 2;
     PeakRec* recs = reinterpret_cast<PeakRec*>(list);
     TTM_CUDA_TRY(cudaMemsetAsync(n_cand, 0, 2 * sizeof(int), st));
-    const dim3 grid((unsigned)((X + 31) / 32), (unsigned)((Y + 7) / 8), (unsigned)((Z + kWalk - 1) / kWalk));
-    if (grid.y > 65535u || grid.z > 65535u) return TTM_ERR_UNSUPPORTED;
+    // fewer than 2^31 voxels in boxes of 3^3 and more: the blocks fit one extent
+    const unsigned grid = (unsigned)((X + 31) / 32) * (unsigned)((Y + 7) / 8) * (unsigned)((Z + kWalk - 1) / kWalk);
     peak_candidates_kernel<<<grid, 256, 0, st>>>(score, X, Y, Z, radius, thr, cand, n_cand, cells);
     TTM_TRY(after_launch(cnt));
     if (radius <= 1) {                                   // the first pass took the whole cube

@@ -289,3 +289,29 @@ def test_direct_statistics_beside_values_that_are_not_finite(ttm, value):
     assert keep.sum() > 20000
     assert np.all(w[touched] == 0)
     assert (np.abs(w[keep] - w_o[keep]) / w_o[keep]).max() <= 1e-5
+
+
+@pytest.mark.parametrize("shape", [(5, 600000, 5), (1100000, 5, 5)])
+def test_peaks_of_long_axes(ttm, shape):
+    """Maps longer in y or z than a launch grid's second and third extent of
+    blocks; planted scores, some on both sides of that length."""
+    import torch
+    Z, Y, X = shape
+    t = synth.blob_template(5, 3, seed=1)
+    comp, desc = ttm.build_template(t, synth.ball_mask(5, 2), 2,
+                                    synth.super_fibonacci_quaternions(10).astype(np.float32))
+    m = ttm.Matcher([(comp, desc, synth.ball_mask(5, 2))], [((X, Y, Z), 0)])
+    score = torch.zeros(shape, device="cuda")
+    quat = torch.zeros(shape + (4,), device="cuda")
+    at = [0, 7, 65535, 524279, 524280, 524288, 599999] + ([] if Z < Y else [1048559, 1048560, 1099999])
+    flat = []
+    for k, p in enumerate(at):
+        v = (2 * Y + p) * X + 2 if Z < Y else (p * Y + 2) * X + 2
+        score.view(-1)[v] = 1.0 + k
+        flat.append((p, v, 1.0 + k))
+    for radius in (0, 1, 3, 6):
+        got = ttm.ttm_extract_peaks(m.plan, 0, score, quat, score, 0.5, radius, 100, m.ws)
+        expect = [v for p, v, s in sorted(flat, key=lambda e: -e[2])
+                  if not any(abs(p - p2) <= radius and s2 > s for p2, _, s2 in flat)]
+        assert ((got["z"].astype(np.int64) * Y + got["y"]) * X + got["x"]).tolist() == expect
+    m.close()
