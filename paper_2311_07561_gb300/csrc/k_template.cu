@@ -311,10 +311,11 @@ __global__ void __launch_bounds__(256) cells_kernel(const float* __restrict__ t,
     cells[e] = make_float4(at(x, y), at(x + 1, y), at(x, y + 1), at(x + 1, y + 1));
 }
 
-// s + e = a + b exactly
+// s + e = a + b exactly.  Additions by name, here and for the squares: one that
+// the compiler fuses with the product before it sums something else.
 __device__ __forceinline__ float two_sum(float a, float b, float& e) {
-    const float s = a + b, bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
     return s;
 }
 
@@ -322,9 +323,10 @@ __device__ __forceinline__ float two_sum(float a, float b, float& e) {
 __host__ __device__ constexpr size_t rot_pitch(int n) { return ((size_t)n + 3) & ~(size_t)3; }
 
 // One CTA per node: raw samples of the listed voxels, and the node's offset
-// and scale.  FP64 runs at 1/64 of the FP32 rate here, so the sums of four
-// samples (and of their exact squares) are formed in FP32 without error, sum
-// and remainder apart, and one FP64 addition takes the sum.
+// and scale.  FP64 runs at 1/64 of the FP32 rate here, so four samples (and
+// their squares) are summed in FP32, every addition's and product's remainder
+// kept; one FP64 addition takes the sum, and the remainders, 2^-24 of the sums,
+// add up in FP32 (a rounding of 2^-48).
 __global__ void __launch_bounds__(640, 2) rotate_list_kernel(
     const float4* __restrict__ cells, const float* __restrict__ m, int s,
     const float* __restrict__ quats, int j0, const int* __restrict__ list, int n, int soft,
@@ -376,7 +378,7 @@ __global__ void __launch_bounds__(640, 2) rotate_list_kernel(
                 acc += (az * ay * ax) * hi.w;
                 o[i] = acc;
                 v[k] = acc;
-                a[k] = soft ? __ldg(m + unpack_voxel(p, s)) * acc : acc;
+                a[k] = soft ? __fmul_rn(__ldg(m + unpack_voxel(p, s)), acc) : acc;
             }
         }
         float ea, eb, ec, q[4], r = 0.f;
@@ -385,7 +387,7 @@ __global__ void __launch_bounds__(640, 2) rotate_list_kernel(
         e1 += (ea + eb) + ec;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            q[k] = a[k] * v[k];
+            q[k] = __fmul_rn(a[k], v[k]);
             r += fmaf(a[k], v[k], -q[k]);
         }
         const float s2 = two_sum(two_sum(q[0], q[1], ea), two_sum(q[2], q[3], eb), ec);

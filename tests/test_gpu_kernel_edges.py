@@ -315,3 +315,21 @@ def test_peaks_of_long_axes(ttm, shape):
                   if not any(abs(p - p2) <= radius and s2 > s for p2, _, s2 in flat)]
         assert ((got["z"].astype(np.int64) * Y + got["y"]) * X + got["x"]).tolist() == expect
     m.close()
+
+
+@pytest.mark.parametrize("s,n_rot", [(12, 40), (33, 90)])
+@pytest.mark.parametrize("offset", [30.0, 1e4])
+def test_template_build_far_from_zero(ttm, s, n_rot, offset):
+    """A template on a large offset: its mean and variance under the mask come
+    from sums that nearly cancel.  A sample is eight products and sums in FP32
+    (weights of three factors), at most 12 roundings of the largest value, and
+    the mean carries the same, on top of the bound for a template near zero."""
+    t = (synth.blob_template(s, 4, seed=s).astype(np.float64) + offset).astype(np.float32)
+    mask = synth.ball_mask(s, (s - 1) // 2 - 1)          # samples outside the box would be zero
+    q = synth.super_fibonacci_quaternions(n_rot).astype(np.float32)
+    comp, _ = ttm.build_template(t, mask, 4, q)
+    T = o.tensor_template(t, mask, q.astype(np.float64), np.full(n_rot, 1.0 / n_rot), 4)
+    scale = max(np.abs(o.rotated_normalised(t, mask, v)).max() for v in q[:8].astype(np.float64))
+    spread = np.ptp(t[mask > 0]).astype(np.float64)
+    bound = 2e-5 * np.abs(T).max() + 24 * 2.0 ** -24 * np.abs(t).max() * scale / spread * 2
+    assert np.abs(comp.cpu().numpy() - T).max() <= bound
