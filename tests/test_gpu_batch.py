@@ -265,3 +265,23 @@ def test_host_stream_with_shared_volume_copies(ttm, many):
             assert torch.equal(lo, ref[3 * n + p].cpu()), (k, p)
     hs.close()
     m.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "mixed"])
+@pytest.mark.parametrize("chunks", [3, 8])
+def test_several_waves_in_several_chunks(ttm, many, precision, chunks):
+    """Several resident waves whose search and refinement run chunk by chunk on
+    the two rotation streams, against one problem at a time in one chunk."""
+    tm, pb, vols = many["tmpls"], many["problems"], many["vols"]
+    maps = []
+    for batch_mib, n in ((0, 1), (40, chunks)):
+        po = ttm.PlanOpts()
+        po.precision = ttm.TTM_PREC_FP32 if precision == "fp32" else ttm.TTM_PREC_MIXED
+        po.batch_mib, po.rotation_chunks = batch_mib, n
+        m = ttm.Matcher(tm, pb, opts=po)
+        if batch_mib:
+            assert len(ttm.ttm_plan_waves(m.plan)) >= 2
+        maps.append(_maps(ttm, m, vols))
+        m.close()
+    for p, (a, b) in enumerate(zip(*maps)):
+        assert torch_equal(a, b), p
