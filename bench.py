@@ -114,17 +114,19 @@ NCU_TRAFFIC: dict = {
     # whole interior: the 128^3 case (c2s), 912 673 interior voxels, FP32 maps;
     # the 256x256x192 case of the order-6 template (c5s), 4 805 121 interior
     # voxels, bf16 maps.
-    "rotation_polish": [dict(bytes_per_voxel=(193203200 + 9803008) / 912673, K=35, storage="f32",
-                             source_sha="912e1275591c",
-                             sources=["k_rotation.cuh", "k_rotation.cu", "k_rotation_n4.cu"]),
-                        dict(bytes_per_voxel=(1193875456 + 90971136) / 4805121, K=84,
-                             storage="bf16", source_sha="e2173a68ccde",
-                             sources=["k_rotation.cuh", "k_rotation.cu", "k_rotation_n6.cu"])],
-    "rotation_search": [dict(bytes_per_voxel=(173863936 + 11920384) / 912673, K=35, storage="f32",
-                             source_sha="7ea2aa611a47",
+    "rotation_polish": [dict(bytes_per_voxel=(193264896 + 14254080) / 912673, K=35, storage="f32",
+                             source_sha="270c638ef012",
+                             sources=["k_rotation.cuh", "ttm_f2.cuh", "k_rotation.cu",
+                                      "k_rotation_n4.cu"]),
+                        dict(bytes_per_voxel=(1193854000 + 94209000) / 4805121, K=84,
+                             storage="bf16", source_sha="2ca581964643",
+                             sources=["k_rotation.cuh", "ttm_f2.cuh", "k_rotation.cu",
+                                      "k_rotation_n6.cu"])],
+    "rotation_search": [dict(bytes_per_voxel=(173834752 + 12940544) / 912673, K=35, storage="f32",
+                             source_sha="dabc461ce57e",
                              sources=["k_search_tc.cu", "k_rotation.cuh"]),
-                        dict(bytes_per_voxel=(1094127360 + 91662592) / 4805121, K=84,
-                             storage="bf16", source_sha="7ea2aa611a47",
+                        dict(bytes_per_voxel=(1094204000 + 92230000) / 4805121, K=84,
+                             storage="bf16", source_sha="dabc461ce57e",
                              sources=["k_search_tc.cu", "k_rotation.cuh"])],
 }
 
@@ -608,7 +610,10 @@ def roofline(kernels: dict, steps: int, geo: dict, peaks: dict) -> dict:
     Work is algorithmic: FLOP for the score + rotation step (the planned a5
     count), bytes for the memory-bound stages (what each pass must read and
     write at the plan's storage precision), never a count of what the kernel
-    happens to execute.  The score + rotation stage is timed by its span
+    happens to execute.  The build does less than the plan (its grid search
+    runs on the tensor cores, its refinement takes refinement_flop_per_voxel),
+    so the stage's fraction can exceed one; tensor_pipe and refinement_alu
+    count the work done.  The score + rotation stage is timed by its span
     (rotation_stage: the wall time of the stage on the launch stream), else as
     the sum of its two kernel classes' CUDA-event times (an upper bound)."""
     K, nvox, n_int = geo["K"], geo["nvox"], geo["n_interior"]

@@ -121,7 +121,7 @@ typedef struct ttm_plan_opts {
     int rotation_chunks; /* split the interior into this many chunks and run  */
                          /* the search of chunk i+1 (high-priority stream)    */
                          /* beside the refinement of chunk i (low priority);  */
-                         /* 0 = default (1): one search, then one refinement     */
+                         /* 0 = default (1): one search, then one refinement  */
     float lowpass_sigma; /* > 0: the volume is prefiltered by a Gaussian of   */
                          /* this sigma (voxels, <= 7.9; ttm_lowpass) inside   */
                          /* ttm_local_stats, ttm_correlate, ttm_match_peaks;  */
@@ -306,9 +306,9 @@ ttm_status ttm_plan_device_status(ttm_plan_t plan, void* d_workspace, size_t wor
  * and forgets them.  Class names come from ttm_kernel_class_name; there are
  * TTM_KERNEL_CLASSES classes.  The last, "rotation_stage", is not a kernel
  * but a span: the wall time of each problem's (or resident wave's)
- * score/rotation stage on the launch stream, with its search and refinement
- * overlapped on the plan's two rotation streams; its launches are counted in
- * their own classes as well. */
+ * score/rotation stage on the launch stream (with rotation_chunks > 1 its
+ * search and refinement overlap on the plan's two rotation streams); its
+ * launches are counted in their own classes as well. */
 #define TTM_KERNEL_CLASSES 13
 ttm_status ttm_plan_enable_timing(ttm_plan_t plan, int enable);
 ttm_status ttm_plan_timing(ttm_plan_t plan, double* ms, long long* launches, int n_classes);
@@ -325,9 +325,10 @@ void ttm_plan_destroy(ttm_plan_t plan);
  *   S1(x) = sum_u m(u) f(x + u - c),  S2(x) = sum_u m(u) f(x + u - c)^2,
  * into d_w[p] (X*Y*Z float32).  w = 0 outside the interior and where the
  * local variance S2 - S1^2/<1,m> is at most 1e-6 * <1,m> * var(f), var(f)
- * being the variance of the whole volume.  S1 and S2 are accumulated in FP32
- * after subtracting a per-tile reference value; the variance is formed in
- * FP64.  d_vols[p] is read, never written.
+ * being the variance of the whole volume.  Direct path: S1 and S2 are FP64
+ * sums after subtracting a per-tile reference value.  FFT path: FP32 window
+ * sums of the volume less its mean, with a bound on their rounding error, and
+ * FP64 sums where that bound is too large.  d_vols[p] is read, never written.
  * Errors: TTM_ERR_INVALID_ARG, TTM_ERR_WORKSPACE, TTM_ERR_CUDA.
  * ---------------------------------------------------------------------- */
 ttm_status ttm_local_stats(ttm_plan_t plan, const float* const* d_vols, float* const* d_w,

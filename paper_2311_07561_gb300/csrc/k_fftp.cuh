@@ -396,7 +396,7 @@ template <int L, typename TS> struct MulPlan {
 // rotated template's box: len planes, the rest zero).  The team transforms a
 // line forward, multiplies, and goes on, the products where the samples were:
 // the template spectra are neither written nor read (128 points, boxes of 24,
-// 501 lines a column: 2152 us of z pass and 2622 of multiply -> 3276).
+// 500 templates: 2152 us of z pass and 2622 of multiply -> 3276).
 // Persistent CTAs over column tiles; the teams of a CTA (L1 NP threads with
 // a named barrier each) share the tile's image samples in shared memory (the
 // next tile's arrive meanwhile) and take the components in turn.
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(L1 * NP * mulp_teams<L1, L2, NP, MS, TS, BOX>(
 // step runs; a thread of the first step reads the samples of its two rows, and
 // their mirrored ones, from there.  HALF: through a complex transform of half
 // the length (rows_c2r_half_t), else of the whole length with the Hermitian
-// extension (rows_c2r2_t).
+// extension.
 constexpr int kRowThreads = 128;
 // row pairs per tile: the first step's items fill the CTA once or twice, the
 // second step's once

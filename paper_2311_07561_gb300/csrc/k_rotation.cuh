@@ -62,10 +62,9 @@ static __device__ __forceinline__ int seg_of(const RotBatch& b, uint32_t t, int 
 }
 
 // The score sum_alpha mu_alpha C_alpha^2 is accumulated in two halves, the
-// components below score_split<N>() and the rest, added at the end: the
-// tensor-core search loads the two halves of a voxel's components in two
-// threads, and every kernel that writes a score map sums in this same order,
-// so the maps agree bit for bit.
+// components below score_split<N>() and the rest, added at the end (two shorter
+// chains): every kernel that writes a score map sums in this same order, so the
+// maps agree bit for bit.
 template <int N>
 __host__ __device__ constexpr int score_split() { return ((n_comp(N) + 1 + 15) / 16) * 8; }
 

@@ -726,11 +726,15 @@ ttm_status launch_build_cells(const TemplateBuild& b, const float* t, cudaStream
 ttm_status launch_build_nodes(const TemplateBuild& b, int n_order, const float* quats,
                               const float* weights, int n_rot, int j0, int nj, float* comp,
                               int* d_bad, cudaStream_t st, long long* cnt) {
-    // small masks: fewer warps to reduce per node; few nodes (the 304 that a
-    // large mask's samples leave room for): two CTAs hold all the threads an SM
-    // takes at 48 registers (64^3 box, order 6, 20000 nodes: 40.9 -> 28.9 ms the
-    // build, against 256 threads); many nodes: 256 (32^3 box, 1024 nodes a
-    // chunk: 963 us of samples, 1061 with 512)
+    // small masks: fewer warps to reduce per node; few nodes (the 304 to 608 that
+    // a box from 39^3 on leaves room for): two CTAs hold all the threads an SM
+    // takes at 48 registers; many nodes: 256.  Builds of order 2, 2400 nodes, ms
+    // with 128 / 256 / 640 threads: 20^3 (3071 voxels) 0.332 / 0.348 / 0.380, 24^3
+    // (5575) 0.356 / 0.365 / 0.400, 28^3 0.455 / 0.448 / 0.462, 36^3 0.821 / 0.673
+    // / 0.723, 40^3 1.15 / 0.845 / 0.812, 48^3 2.56 / 1.60 / 1.16, 64^3 6.34 / 3.73
+    // / 2.28, 127^3 (1000 nodes) 50 / 26.6 / 12.6; 300 nodes: 24^3 0.220 / 0.216 /
+    // 0.203, 32^3 0.260 / 0.230 / 0.207.  384 threads beat 640 at 42^3 and 44^3
+    // (0.873 against 0.987, 1.07 against 1.20), elsewhere from 39^3 on they lose.
     const int threads = b.n < 4096 ? 128 : nj <= 4 * 152 ? 640 : 256;
     rotate_list_kernel<<<nj, threads, 0, st>>>(reinterpret_cast<const float4*>(b.cells), b.mask, b.s,
                                                quats, j0, b.list, b.n, b.soft, b.rot, b.norm,

@@ -506,8 +506,9 @@ constexpr size_t kProdBudget = (size_t)8 << 30;
 int comp_group(const ttm_plan_s* P, const ProblemData& pr) {
     const size_t per = pr.fft.nspec() * 2 * (pr.mixed ? 2 : 4);
     size_t g = per ? kProdBudget / per : (size_t)P->K;
-    // whole rounds of the fused multiply's teams (2 to 8 per CTA take the
-    // components of a group in turn)
+    // whole rounds of the fused multiply's teams, which take the components of a
+    // group in turn, where a CTA has 1, 2, 3, 4 or 6 of them (up to 11
+    // components: 1 or 3)
     if (g < (size_t)P->K) g = g >= 12 ? g / 12 * 12 : g >= 3 ? g / 3 * 3 : g;
     return (int)std::max<size_t>(1, std::min<size_t>(g, (size_t)P->K));
 }
