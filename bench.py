@@ -115,18 +115,18 @@ NCU_TRAFFIC: dict = {
     # the 256x256x192 case of the order-6 template (c5s), 4 805 121 interior
     # voxels, bf16 maps.
     "rotation_polish": [dict(bytes_per_voxel=(193264896 + 14254080) / 912673, K=35, storage="f32",
-                             source_sha="270c638ef012",
+                             source_sha="71e05aa45dde",
                              sources=["k_rotation.cuh", "ttm_f2.cuh", "k_rotation.cu",
                                       "k_rotation_n4.cu"]),
                         dict(bytes_per_voxel=(1193854000 + 94209000) / 4805121, K=84,
-                             storage="bf16", source_sha="2ca581964643",
+                             storage="bf16", source_sha="5bbbaa9eec8b",
                              sources=["k_rotation.cuh", "ttm_f2.cuh", "k_rotation.cu",
                                       "k_rotation_n6.cu"])],
     "rotation_search": [dict(bytes_per_voxel=(173834752 + 12940544) / 912673, K=35, storage="f32",
-                             source_sha="dabc461ce57e",
+                             source_sha="a26fd874e389",
                              sources=["k_search_tc.cu", "k_rotation.cuh"]),
                         dict(bytes_per_voxel=(1094204000 + 92230000) / 4805121, K=84,
-                             storage="bf16", source_sha="dabc461ce57e",
+                             storage="bf16", source_sha="a26fd874e389",
                              sources=["k_search_tc.cu", "k_rotation.cuh"])],
 }
 

@@ -383,6 +383,23 @@ __device__ __forceinline__ F2 f2_dot(const F2 (&a)[4], const F2 (&b)[4]) {
     return f2_fma(a[3], b[3], f2_fma(a[2], b[2], f2_fma(a[0], b[0], f2_mul(a[1], b[1]))));
 }
 
+// Row i of a symmetric matrix times x.  At order 2 the matrix is C itself and the
+// Newton matrix differs from it in the diagonal alone, so the scalar code forms
+// the off-diagonal products of the two once, rounded, and only what one of them
+// has to itself is fused.  (A packed multiplication and the packed addition after
+// it are fused all the same, so a rounded product that is added is scalar.)
+__device__ __forceinline__ F2 f2_round_mul(F2 a, F2 b) {
+    return f2(__fmul_rn(f2_get(a, 0), f2_get(b, 0)), __fmul_rn(f2_get(a, 1), f2_get(b, 1)));
+}
+template <int N>
+__device__ __forceinline__ F2 f2_row(int i, const F2 (&a)[4], const F2 (&b)[4]) {
+    if (N != 2 || i == 3) return f2_dot(a, b);
+    const F2 last = f2_round_mul(a[3], b[3]);
+    if (i == 2) return f2_add(f2_fma(a[2], b[2], f2_fma(a[0], b[0], f2_mul(a[1], b[1]))), last);
+    const F2 s = i == 0 ? f2_fma(a[0], b[0], f2_mul(a[1], b[1])) : f2_fma(a[1], b[1], f2_mul(a[0], b[0]));
+    return f2_add(f2_add(s, f2_round_mul(a[2], b[2])), last);
+}
+
 // the gradient of grad_at for two points (its lam is f2_dot(x, g))
 template <int N>
 __device__ __forceinline__ void grad2_at(const F2 (&C)[Geo<N>::K], const F2 (&x)[4], F2 (&g)[4]) {
@@ -420,7 +437,7 @@ __device__ __forceinline__ void eval2_at(const F2 (&C)[Geo<N>::K], const F2 (&x)
     const F2 H[4][4] = {{h[0], h[1], h[2], h[3]}, {h[1], h[4], h[5], h[6]},
                         {h[2], h[5], h[7], h[8]}, {h[3], h[6], h[8], h[9]}};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) g[i] = f2_dot(H[i], x);
+    for (int i = 0; i < 4; ++i) g[i] = f2_row<N>(i, H[i], x);
     lam = f2_dot(g, x);
 }
 
@@ -471,7 +488,7 @@ __device__ __forceinline__ void newton_dir2(const F2 (&h)[10], const F2 (&g)[4],
         }
     F2 Bx[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) Bx[i] = f2_dot(B[i], x);
+    for (int i = 0; i < 4; ++i) Bx[i] = f2_row<N>(i, B[i], x);
     const F2 cxx = f2_sub(f2_dot(x, Bx), f2(sig, sig));
 #pragma unroll
     for (int i = 0; i < 4; ++i) Bx[i] = f2_mul(Bx[i], minus);

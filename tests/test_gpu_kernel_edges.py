@@ -333,3 +333,23 @@ def test_template_build_far_from_zero(ttm, s, n_rot, offset):
     spread = np.ptp(t[mask > 0]).astype(np.float64)
     bound = 2e-5 * np.abs(T).max() + 24 * 2.0 ** -24 * np.abs(t).max() * scale / spread * 2
     assert np.abs(comp.cpu().numpy() - T).max() <= bound
+
+
+@pytest.mark.parametrize("n", [2, 4, 6])
+def test_bits_of_the_scalar_forms(ttm, n):
+    """w, score, lambda and q at 1500 voxels, to the bit what the scalar FFT
+    passes and the scalar refinement gave before two lines or two candidates
+    shared a register pair (recorded in tests/golden/scalar_passes.npz).  Lines
+    of 144 and 160 points along z and x, of 48 along y."""
+    import os
+    gold = np.load(os.path.join(os.path.dirname(__file__), "golden", "scalar_passes.npz"))
+    shape = (132, 36, 150)
+    wl = synth.make_workload(shape, 9, 3, 2, 1.0, n, 200, radius=4, seeds=(71, 72, 73))
+    comp, desc = ttm.build_template(wl.template, wl.mask, n, wl.quadrature)
+    res, box = _maps(ttm, wl.volume, comp, desc, wl.mask, path=ttm.TTM_PATH_FFT)
+    assert list(box) == [160, 48, 144]
+    inner = tuple(d - 8 for d in shape)
+    at = np.random.default_rng(9).choice(int(np.prod(inner)), 1500, replace=False)
+    z, y, x = (i + 4 for i in np.unravel_index(at, inner))
+    for k in ("w", "score", "lam", "quat"):
+        assert np.array_equal(res[k][z, y, x], gold[f"{k}{n}"]), k
