@@ -1632,7 +1632,7 @@ ttm_status ttm_extract_peaks(ttm_plan_t plan, int problem, const float* d_score,
     float* tmp_b = (float*)(ws + kHeader + align256(nv * sizeof(float)));
     void* list = ws + kHeader + 2 * align256(nv * sizeof(float));
     const int cap = (int)peak_cap(nv);
-    TTM_CUDA_TRY(cudaMemsetAsync(d_count, 0, sizeof(int), st));
+    TTM_CUDA_TRY(cudaMemsetAsync(d_count, 0, 3 * sizeof(int), st));   // peaks, candidates, those left
     TTM_TRY(timed(plan, KC_PEAKS, st, [&] {
         return launch_peak_candidates_full(d_score, d_quat, d_lambda, pr.X, pr.Y, pr.Z, threshold,
                                            radius, tmp_a, tmp_b, list, cap, d_count, st,
@@ -1677,7 +1677,7 @@ ttm_status ttm_match_peaks(ttm_plan_t plan, int problem, const float* d_vol, con
     char* list = pk + 2 * align256(nv * sizeof(float));
     const int cap = (int)peak_cap(nv);
     const VoxBox box = interior_box(pr.X, pr.Y, pr.Z, T.desc.s);
-    TTM_CUDA_TRY(cudaMemsetAsync(ws + 16, 0, 32, st));       // peak count, status word
+    TTM_CUDA_TRY(cudaMemsetAsync(ws + 16, 0, 32, st));       // peak counts, status word
     const float* vol = nullptr;
     TTM_TRY(prefilter(plan, pr, d_vol, d_workspace, st, &vol));
     TTM_TRY(corr_problem(plan, pr, vol, d_workspace, st));

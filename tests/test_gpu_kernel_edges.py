@@ -353,3 +353,40 @@ def test_bits_of_the_scalar_forms(ttm, n):
     z, y, x = (i + 4 for i in np.unravel_index(at, inner))
     for k in ("w", "score", "lam", "quat"):
         assert np.array_equal(res[k][z, y, x], gold[f"{k}{n}"]), k
+
+
+def _peaks_by_rank(score, threshold, radius):
+    """The oracle's peaks (o.extract_peaks) for large cubes: ranks by score and,
+    where equal, by falling index; a peak is the highest rank of its cube."""
+    from scipy.ndimage import maximum_filter1d
+    flat = score.ravel()
+    rank = np.empty(flat.size, dtype=np.int64)
+    rank[np.lexsort((-np.arange(flat.size), flat))] = np.arange(flat.size)
+    best = rank = rank.reshape(score.shape)
+    for axis in range(3):
+        best = maximum_filter1d(best, 2 * radius + 1, axis=axis, mode="constant", cval=-1)
+    idx = np.nonzero(((best == rank) & (score > threshold)).ravel())[0]
+    return idx[np.lexsort((idx, -flat[idx]))]
+
+
+@pytest.mark.parametrize("shape", [(5, 5, 5), (29, 40, 70), (70, 21, 33), (66, 67, 69)])
+@pytest.mark.parametrize("levels", [1, 2, 4, 10 ** 6])
+def test_peaks_of_large_cubes(ttm, shape, levels):
+    """Cubes that hold many cells, up to the largest radius, in maps with a few
+    levels (equal scores in whole cells) and with none alike."""
+    Z, Y, X = shape
+    rng = np.random.default_rng(Y)
+    mask = synth.ball_mask(5, 2)
+    comp, desc = ttm.build_template(synth.blob_template(5, 3, seed=1), mask, 2,
+                                    synth.super_fibonacci_quaternions(10).astype(np.float32))
+    m = ttm.Matcher([(comp, desc, mask)], [((X, Y, Z), 0)])
+    quat = np.zeros(shape + (4,), dtype=np.float32)
+    score = (np.floor(rng.random(shape) * levels) / levels + 0.25).astype(np.float32)
+    if shape == (5, 5, 5):
+        assert np.array_equal(_peaks_by_rank(score, 0.2, 3), o.extract_peaks(score.astype(np.float64), 0.2, 3, 125))
+    for radius in (5, 6, 9, 13, 20, 32):
+        got = ttm.ttm_extract_peaks(m.plan, 0, _cuda(score), _cuda(quat), _cuda(score), 0.2,
+                                    radius, score.size, m.ws)
+        expect = _peaks_by_rank(score, 0.2, radius)
+        assert np.array_equal((got["z"].astype(np.int64) * Y + got["y"]) * X + got["x"], expect)
+    m.close()
