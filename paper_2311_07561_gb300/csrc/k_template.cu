@@ -33,20 +33,34 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
     return red[0];
 }
 
+// <1, m> by one CTA of kRotThreads threads or more (the order of the sum is part
+// of the result; further threads add nothing).  16 loads in flight, then 4, then
+// one: an FP64 addition costs its 16 clocks a warp also where a predicate skips it
+template <int G>
+__device__ __forceinline__ void mask_add(const float* __restrict__ m, int n, int& i, double& acc) {
+    for (; i + (G - 1) * kRotThreads < n; i += G * kRotThreads) {
+        float v[G];
+#pragma unroll
+        for (int k = 0; k < G; ++k) v[k] = __ldg(m + i + k * kRotThreads);
+#pragma unroll
+        for (int k = 0; k < G; ++k)
+            if (v[k] != 0.f) acc += (double)v[k];
+    }
+}
+
+__device__ __forceinline__ double mask_sum(const float* __restrict__ m, int n, double* red) {
+    double acc = 0.0;
+    int i = threadIdx.x < kRotThreads ? threadIdx.x : n;
+    mask_add<16>(m, n, i, acc);
+    mask_add<4>(m, n, i, acc);
+    mask_add<1>(m, n, i, acc);
+    return block_sum(acc, red);
+}
+
 __global__ void __launch_bounds__(kRotThreads) mask_sum_kernel(const float* __restrict__ m,
                                                                int n, double* out) {
     __shared__ double red[32];
-    double acc = 0.0;
-    // one CTA (the order of the sum is part of the result): 16 loads in flight
-    for (int i0 = threadIdx.x; i0 < n; i0 += 16 * kRotThreads) {
-        float v[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = i0 + k * kRotThreads < n ? __ldg(m + i0 + k * kRotThreads) : 0.f;
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if (v[k] != 0.f) acc += (double)v[k];
-    }
-    double s = block_sum(acc, red);
+    const double s = mask_sum(m, n, red);
     if (threadIdx.x == 0) *out = s;
 }
 
@@ -241,6 +255,7 @@ struct VoxelList {            // what the prepass leaves in the workspace header
     int n;                    // mask voxels
     int odd;                  // template or mask values that are not finite
     int soft;                 // mask values other than 0 and 1
+    int summed;               // mask_sum holds the sum of a soft mask
 };
 
 __device__ __forceinline__ int brick_voxel(int e, int s) {     // packed x | y << 8 | z << 16, or -1
@@ -255,12 +270,34 @@ __device__ __forceinline__ int unpack_voxel(int p, int s) {
 }
 
 constexpr int kListThreads = 1024;
+// boxes up to this edge: a CTA more sums the mask where it is soft, beside the
+// ones that count, so that the host need not wait twice (order 4, 50 nodes: 24^3
+// 111 -> 94 us, all voxels 95; 32^3 136 -> 117); a larger mask would take that CTA
+// longer than the wait
+constexpr int kListSumEdge = 32;
 
 // mask voxels per CTA of brick-ordered positions; the flags of VoxelList
 __global__ void __launch_bounds__(kListThreads) list_count_kernel(const float* __restrict__ t,
                                                                   const float* __restrict__ m, int s,
-                                                                  int* __restrict__ counts,
+                                                                  int* __restrict__ counts, int blocks,
                                                                   VoxelList* __restrict__ out) {
+    if ((int)blockIdx.x == blocks) {
+        __shared__ double red[32];
+        const int n = s * s * s;
+        bool any = false;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < n; i += kListThreads) {
+            const float v = __ldg(m + i);
+            any = any || (v != 0.f && v != 1.f);
+        }
+        if (!__syncthreads_or(any)) return;
+        const double sum = mask_sum(m, n, red);
+        if (threadIdx.x == 0) {
+            out->mask_sum = sum;
+            out->summed = 1;
+        }
+        return;
+    }
     const int p = brick_voxel(blockIdx.x * kListThreads + threadIdx.x, s);
     const float mv = p >= 0 ? m[unpack_voxel(p, s)] : 0.f;
     const float tv = p >= 0 ? t[unpack_voxel(p, s)] : 0.f;
@@ -675,22 +712,34 @@ ttm_status launch_build_prepass(const float* t, const float* m, int s, void* hea
     VoxelList* vl = reinterpret_cast<VoxelList*>(head);
     const int nb = list_blocks(s);
     int* counts = reinterpret_cast<int*>(area + area_floats - nb);
-    list_count_kernel<<<nb, kListThreads, 0, st>>>(t, m, s, counts, vl);
+    list_count_kernel<<<nb + (s <= kListSumEdge ? 1 : 0), kListThreads, 0, st>>>(t, m, s, counts, nb, vl);
     TTM_TRY(after_launch(cnt));
     list_write_kernel<<<nb, kListThreads, 0, st>>>(m, s, counts, reinterpret_cast<int*>(area), vl);
     return after_launch(cnt);
 }
 
-// The prepass needs the list and its counts side by side in the area.
-bool build_prepass_fits(int s, size_t area_floats) {
-    return area_floats >= (size_t)s * s * s + (size_t)list_blocks(s);
+// Whether the build goes over listed voxels, as far as that can be said before
+// they are counted.  The prepass needs the list and its counts side by side in
+// the area, the layout its tables.  A small box with few nodes is folded before
+// the list is made: its prepass and further launches take 8 to 15 us, and the box
+// build's time grows by 0.09, 0.1, 0.22 and 0.4 us a node at orders 2, 4, 6 and 8
+// (us of the call, all voxels / listed: order 2, 10^3, 300 nodes 84 / 89, 600 117 /
+// 106; order 4, 10^3, 150 80 / 88, 200 94 / 85; order 6, 8^3, 30 77 / 70; order 8,
+// 8^3, 10 93 / 103, 30 94 / 76).  From 24^3 on the list costs no more than the mask
+// sum that it saves (order 4, 24^3, 10 nodes 92 / 94, 50 95 / 88; 32^3, 10 155 / 142).
+bool build_takes_list(int s, int n_order, int n_rot, int nj, size_t area_floats) {
+    if (area_floats < (size_t)s * s * s + (size_t)list_blocks(s)) return false;
+    const size_t side = (size_t)s + 3;
+    if (4 * side * side * (side + 1) + (size_t)nj * (fold_row(n_comp(n_order)) + 2 + 4) > area_floats) return false;
+    const int least = n_order == 2 ? 400 : n_order == 4 ? 180 : n_order == 6 ? 40 : 20;
+    return s >= 24 || n_rot >= least;
 }
 
-// The sum of a binary, finite mask from the prepass; false for another.
+// The sum of a finite mask from the prepass, where it has one.
 bool build_mask_count(const void* head_host, double* mask_sum) {
     const VoxelList& vl = *reinterpret_cast<const VoxelList*>(head_host);
-    if (vl.odd || vl.soft) return false;
-    *mask_sum = (double)vl.n;
+    if (vl.odd || (vl.soft && !vl.summed)) return false;
+    *mask_sum = vl.soft ? vl.mask_sum : (double)vl.n;
     return true;
 }
 

@@ -1146,7 +1146,7 @@ ttm_status ttm_build_tensor_template(const float* d_template, const float* d_mas
     // tables beside the rotated copies (the copies shrink by the voxels left
     // out), else every voxel of the box
     const size_t area = (size_t)nj * s3;
-    const bool prepass = build_prepass_fits(s, area);
+    const bool prepass = build_takes_list(s, n_order, n_rot, nj, area);
     if (prepass)
         TTM_TRY(launch_build_prepass(d_template, d_mask, s, ws, rot, area, st, &cnt));
     else

@@ -323,7 +323,7 @@ struct TemplateBuild {
     float* coef = nullptr;                // w_j q_j^alpha per node
     float* rot = nullptr;                 // samples, n per node
 };
-bool build_prepass_fits(int s, size_t area_floats);
+bool build_takes_list(int s, int n_order, int n_rot, int nj, size_t area_floats);
 ttm_status launch_build_prepass(const float* t, const float* m, int s, void* head, float* area,
                                 size_t area_floats, cudaStream_t st, long long* cnt);
 bool build_mask_count(const void* head_host, double* mask_sum);

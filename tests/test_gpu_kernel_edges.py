@@ -390,3 +390,29 @@ def test_peaks_of_large_cubes(ttm, shape, levels):
         expect = _peaks_by_rank(score, 0.2, radius)
         assert np.array_equal((got["z"].astype(np.int64) * Y + got["y"]) * X + got["x"], expect)
     m.close()
+
+
+@pytest.mark.parametrize("s,n,n_rot,kind,scale", [
+    (6, 4, 180, "ball", 1.0), (6, 4, 179, "ball", 1.0),      # either side of the node count
+    (10, 2, 400, "scattered", 1.0), (10, 2, 399, "scattered", 1.0),
+    (9, 6, 40, "lopsided", 1.0), (9, 8, 20, "ball", 1.0),
+    (3, 2, 700, "full", 1.0), (4, 6, 300, "ball", 1.0),      # no room for the tables
+    (13, 4, 200, "soft", 1.0), (32, 2, 20, "soft", 1.0), (33, 2, 20, "soft", 1.0),
+    (23, 4, 20, "ball", 1.0), (24, 4, 20, "ball", 1.0),      # either side of the edge
+    (12, 4, 200, "ball", 1e-25), (12, 4, 200, "ball", 1e20),
+])
+def test_template_build_of_both_forms(ttm, s, n, n_rot, kind, scale):
+    """Boxes and node counts on both sides of the line between the build over
+    every voxel and the one over the mask's, and soft masks summed by either."""
+    t = (synth.blob_template(s, 4, seed=s).astype(np.float64) * scale).astype(np.float32)
+    if kind == "soft":
+        mask = synth.soft_ball_mask(s, s // 2, 2.0)
+    else:
+        mask = np.ones((s, s, s), np.float32) if kind == "full" else _mask(kind, s)
+    q = synth.super_fibonacci_quaternions(n_rot).astype(np.float32)
+    w = np.random.default_rng(s).random(n_rot).astype(np.float32)
+    w /= w.sum()
+    comp, desc = ttm.build_template(t, mask, n, q, weights=w)
+    T = o.tensor_template(t, mask, q.astype(np.float64), w.astype(np.float64), n)
+    assert desc.mask_sum == pytest.approx(mask.sum(dtype=np.float64))
+    assert np.abs(comp.cpu().numpy() - T).max() <= 2e-5 * np.abs(T).max()
