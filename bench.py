@@ -123,10 +123,10 @@ NCU_TRAFFIC: dict = {
                              sources=["k_rotation.cuh", "ttm_f2.cuh", "k_rotation.cu",
                                       "k_rotation_n6.cu"])],
     "rotation_search": [dict(bytes_per_voxel=(173834752 + 12940544) / 912673, K=35, storage="f32",
-                             source_sha="a26fd874e389",
+                             source_sha="297fbfaecf99",
                              sources=["k_search_tc.cu", "k_rotation.cuh"]),
                         dict(bytes_per_voxel=(1094204000 + 92230000) / 4805121, K=84,
-                             storage="bf16", source_sha="a26fd874e389",
+                             storage="bf16", source_sha="297fbfaecf99",
                              sources=["k_search_tc.cu", "k_rotation.cuh"])],
 }
 

@@ -101,8 +101,12 @@ constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kChunkN >> 3) << 17) | ((128
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase) {
     return mbar_wait_bounded(bar, phase, kMbarWaitPolls);
 }
-// the same by all lanes of a warp, with one answer for all of them
+// The same by all lanes of a warp, with one answer for all of them.  The vote on
+// a first poll keeps the loop, whose lanes may part, off the usual path (search of
+// the 256^3 case: 3.51 ms, 3.57 with a vote after the loop alone, 3.51 without
+// votes).
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t phase) {
+    if (__all_sync(0xffffffffu, mbar_wait_bounded(bar, phase, 1))) return true;
     return __all_sync(0xffffffffu, mbar_wait(bar, phase));
 }
 
