@@ -115,18 +115,18 @@ NCU_TRAFFIC: dict = {
     # the 256x256x192 case of the order-6 template (c5s), 4 805 121 interior
     # voxels, bf16 maps.
     "rotation_polish": [dict(bytes_per_voxel=(193264896 + 14254080) / 912673, K=35, storage="f32",
-                             source_sha="71e05aa45dde",
+                             source_sha="beec3033726e",
                              sources=["k_rotation.cuh", "ttm_f2.cuh", "k_rotation.cu",
                                       "k_rotation_n4.cu"]),
                         dict(bytes_per_voxel=(1193854000 + 94209000) / 4805121, K=84,
-                             storage="bf16", source_sha="5bbbaa9eec8b",
+                             storage="bf16", source_sha="a250474ba4a8",
                              sources=["k_rotation.cuh", "ttm_f2.cuh", "k_rotation.cu",
                                       "k_rotation_n6.cu"])],
     "rotation_search": [dict(bytes_per_voxel=(173834752 + 12940544) / 912673, K=35, storage="f32",
-                             source_sha="297fbfaecf99",
+                             source_sha="8ae830a58322",
                              sources=["k_search_tc.cu", "k_rotation.cuh"]),
                         dict(bytes_per_voxel=(1094204000 + 92230000) / 4805121, K=84,
-                             storage="bf16", source_sha="297fbfaecf99",
+                             storage="bf16", source_sha="8ae830a58322",
                              sources=["k_search_tc.cu", "k_rotation.cuh"])],
 }
 

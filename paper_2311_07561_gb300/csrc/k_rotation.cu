@@ -10,7 +10,7 @@ static void fill_args(const RotBatch& b, const RotGrid& g, rot::SearchArgs& sa,
     sa.b = b; pa.b = b;
     sa.list = list; pa.list = list;
     sa.gm = g.d_m; sa.cell_end = g.d_cell_end; sa.n_grid = g.n_grid; sa.n_cand = g.n_cand;
-    pa.gq = g.d_q; pa.n_cand = g.n_cand; pa.newton = g.newton; pa.n_refine = g.n_refine;
+    pa.gq = g.d_q; pa.n_grid = g.n_grid; pa.n_cand = g.n_cand; pa.newton = g.newton; pa.n_refine = g.n_refine;
 }
 
 // a batch's units lie in their problems' interiors; unit lists serve one problem

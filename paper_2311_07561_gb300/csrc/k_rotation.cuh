@@ -51,6 +51,8 @@ struct PolishArgs {
     UnitList list;          // optional unit list (peaks) and strided outputs
     const float* gq;        // n_grid x 4
     int n_cand, newton, n_refine;
+    int n_grid;             // a candidate from n_grid up is none: 0xFFFF, or what a
+                            // search that gave up has left unwritten
 };
 
 static_assert(kRotThreads == kRotTile, "one block of the SIMT kernels is one tile");
@@ -640,9 +642,9 @@ __device__ __forceinline__ void polish_pairs(const float (&Cs)[Geo<N>::K4], floa
     for (int k = 0; k < nc; k += 2) {
         const uint32_t pair = k < 4 ? (k < 2 ? cw[0] : cw[1]) : (k < 6 ? cw[2] : cw[3]);
         const int ia = (int)(pair & 0xFFFFu);
-        if (ia == 0xFFFF) break;
+        if (ia >= a.n_grid) break;
         int ib = (int)(pair >> 16);
-        const bool two = k + 1 < nc && ib != 0xFFFF;
+        const bool two = k + 1 < nc && ib < a.n_grid;
         if (!two) ib = ia;
         F2 x[4], lam;
 #pragma unroll
@@ -790,7 +792,7 @@ __global__ void __launch_bounds__(kRotThreads, polish_ctas<N>()) polish_kernel(c
     const uint32_t cw[4] = {cr.x, cr.y, cr.z, cr.w};
     float best_l = 0.f;
     float best_q[4] = {1.f, 0.f, 0.f, 0.f};
-    if (score > 0.f && (cw[0] & 0xFFFFu) != 0xFFFFu) {
+    if (score > 0.f && (int)(cw[0] & 0xFFFFu) < a.n_grid) {
         if constexpr (kPairs<N>) {
             polish_pairs<N>(C, score, cw, a, best_l, best_q);
         } else {
@@ -811,7 +813,7 @@ __global__ void __launch_bounds__(kRotThreads, polish_ctas<N>()) polish_kernel(c
 #pragma unroll 1
         for (int k = 0; k < a.n_cand && k < kMaxCand; ++k) {
             const int gi = (int)((cw[k >> 1] >> (16 * (k & 1))) & 0xFFFFu);
-            if (gi == 0xFFFF) break;
+            if (gi >= a.n_grid) break;
             float x[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) x[i] = __ldg(a.gq + 4 * gi + i);

@@ -68,3 +68,16 @@ def test_row_pass_counts_a_copy_it_gave_up_on_as_in_flight():
     assert "bar_wait(" in kernel[wait + 30:left], "no second wait"
     assert not re.search(r"pending &=|phase \^=", kernel[wait:left])
     assert re.search(r"pending &= ~", kernel[left:]) and re.search(r"phase \^=", kernel[left:])
+
+
+def test_refinement_reads_only_grid_points():
+    """A search that gave up leaves candidates unwritten, and the refinement is
+    queued behind it: what is no index of the grid counts as no candidate, not
+    only the mark for none."""
+    text = open(os.path.join(os.path.dirname(SEARCH), "k_rotation.cuh")).read()
+    text = re.sub(r"//[^\n]*", "", text)
+    assert not re.search(r"[=!]= 0xFFFF", text)
+    reads = re.findall(r"a\.gq \+ 4 \* (\w+)", text)
+    assert sorted(set(reads)) == ["gi", "ia", "ib"]
+    for index in set(reads):
+        assert re.search(rf"\b{index} (?:>=|<) a\.n_grid", text), index
