@@ -114,18 +114,18 @@ NCU_TRAFFIC: dict = {
     # whole interior: the 128^3 case (c2s), 912 673 interior voxels, FP32 maps;
     # the 256x256x192 case of the order-6 template (c5s), 4 805 121 interior
     # voxels, bf16 maps.
-    "rotation_polish": [dict(bytes_per_voxel=(193264896 + 14254080) / 912673, K=35, storage="f32",
+    "rotation_polish": [dict(bytes_per_voxel=(193247232 + 13905152) / 912673, K=35, storage="f32",
                              source_sha="beec3033726e",
                              sources=["k_rotation.cuh", "ttm_f2.cuh", "k_rotation.cu",
                                       "k_rotation_n4.cu"]),
-                        dict(bytes_per_voxel=(1193854000 + 94209000) / 4805121, K=84,
+                        dict(bytes_per_voxel=(1193858000 + 94389504) / 4805121, K=84,
                              storage="bf16", source_sha="a250474ba4a8",
                              sources=["k_rotation.cuh", "ttm_f2.cuh", "k_rotation.cu",
                                       "k_rotation_n6.cu"])],
-    "rotation_search": [dict(bytes_per_voxel=(173834752 + 12940544) / 912673, K=35, storage="f32",
+    "rotation_search": [dict(bytes_per_voxel=(173957120 + 13089536) / 912673, K=35, storage="f32",
                              source_sha="8ae830a58322",
                              sources=["k_search_tc.cu", "k_rotation.cuh"]),
-                        dict(bytes_per_voxel=(1094204000 + 92230000) / 4805121, K=84,
+                        dict(bytes_per_voxel=(1094444000 + 92248576) / 4805121, K=84,
                              storage="bf16", source_sha="8ae830a58322",
                              sources=["k_search_tc.cu", "k_rotation.cuh"])],
 }
